@@ -3,6 +3,7 @@
 // and populations cross the boundary in fp64; the arithmetic is fp64 except
 // where k_init_eq and k_moments state otherwise for fp32 and 16-bit storage.
 #include "aux.cuh"
+#include "field_math.cuh"
 #include "internal.h"
 
 namespace fpc {
@@ -42,67 +43,19 @@ static AlphaMap alpha_map()
 // only small terms are summed.  (Equal to C(u)^-1 kappa^eq with kappa^eq the
 // Maxwellian central moments (1, 0, cs^2) per axis.)
 //
-// The arithmetic follows the storage type.  This GPU's fp64 pipe is a small
-// fraction of its fp32 one, and the fp64 form below took ~220 fp64
-// instructions per cell, which made the kernel fp64-bound (5.7 ms for 256^3)
-// rather than bound by reading the fields.  FP64 storage keeps it.  FP32
-// storage forms the three per-axis factors w1 + dphi in fp64 and then
-// g = rho X Y Z - w with one fma per slot: the cancellation against w costs at
-// most ~8 of fp64's 53 bits, far below the 24 bits stored.  16-bit storage
-// evaluates the expanded form in fp32 (a few fp32 ulps of error against at
-// most 11 stored bits).
+// The arithmetic follows the storage type.  FP64 storage evaluates the expanded form in fp64.
+// 16-bit storage evaluates it in fp32 (a few fp32 ulps of error against at most 11 stored bits).
+// FP32 storage needs every deviation rounded once from more than fp32: it evaluates
+//   g = [dr (A+a) + a] (B+b)(C+c) + A [b (C+c) + B c]
+// on numbers that are sums of two fp32 values (field_math.cuh), two cells per thread on the packed
+// fp32 pipe (k_init_eq_pair), about 400 instructions per cell.  The fp64 form it replaces (the three factors in
+// fp64, one fp64 fma and one conversion per slot, about 110 slots of the fp64 pipe) was bound by
+// that pipe: 3.24 ms for 256^3 cells against 0.46 ms now (2.3 GB of traffic: 0.35 ms).
 template <typename S>
-__global__ void k_init_eq(BoxGeom b, const double* rho, const double* ux, const double* uy, const double* uz,
-                          unsigned c0, unsigned n)
+__device__ __forceinline__ void init_cell_fp64(const BoxGeom& b, unsigned cell, double r, double u0, double u1,
+                                               double u2)
 {
-    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const unsigned cell = c0 + i;
-    if constexpr (std::is_same<S, float>::value) {
-        const double r = rho[i], u[3] = {ux[i], uy[i], uz[i]};
-        double X[3][3];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const double v = u[d], v2 = v * v;
-            X[d][0] = w1(0) + 0.5 * (v2 - v);
-            X[d][1] = w1(1) - v2;
-            X[d][2] = w1(2) + 0.5 * (v2 + v);
-        }
-        float* buf = static_cast<float*>(b.buf);
-#pragma unroll
-        for (int iz = 0; iz < 3; ++iz)
-#pragma unroll
-            for (int iy = 0; iy < 3; ++iy) {
-                const double yz = X[1][iy] * X[2][iz];
-#pragma unroll
-                for (int ix = 0; ix < 3; ++ix) {
-                    const int s = ix + 3 * iy + 9 * iz;
-                    buf[(size_t)s * b.stride + cell] = (float)(r * (X[0][ix] * yz) - wslot(s));
-                }
-            }
-        return;
-    } else if constexpr (!std::is_same<S, double>::value) {
-        const float dr = (float)(rho[i] - 1.0), u[3] = {(float)ux[i], (float)uy[i], (float)uz[i]};
-        float dphi[3][3];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const float v = u[d], v2 = v * v;
-            dphi[d][0] = 0.5f * (v2 - v);
-            dphi[d][1] = -v2;
-            dphi[d][2] = 0.5f * (v2 + v);
-        }
-        S* buf = static_cast<S*>(b.buf);
-#pragma unroll
-        for (int s = 0; s < 27; ++s) {
-            const int ix = s % 3, iy = (s / 3) % 3, iz = s / 9;
-            const float A = (float)w1(ix), B = (float)w1(iy), C = (float)w1(iz);
-            const float a = dphi[0][ix], bb = dphi[1][iy], c = dphi[2][iz];
-            const float dprod = a * (B + bb) * (C + c) + A * (bb * (C + c) + B * c);
-            Store<S>::st(buf + (size_t)s * b.stride + cell, dr * ((A + a) * (B + bb) * (C + c)) + dprod);
-        }
-        return;
-    }
-    const double r = rho[i], u[3] = {ux[i], uy[i], uz[i]};
+    const double u[3] = {u0, u1, u2};
     double dphi[3][3];
     for (int d = 0; d < 3; ++d) {
         const double v = u[d], v2 = v * v;
@@ -122,13 +75,93 @@ __global__ void k_init_eq(BoxGeom b, const double* rho, const double* ux, const 
     }
 }
 
+// FP64 and 16-bit storage, one cell per thread.
+template <typename S>
+__global__ void k_init_eq(BoxGeom b, const double* rho, const double* ux, const double* uy, const double* uz,
+                          unsigned c0, unsigned n)
+{
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const unsigned cell = c0 + i;
+    if constexpr (std::is_same<S, double>::value) {
+        init_cell_fp64<S>(b, cell, rho[i], ux[i], uy[i], uz[i]);
+    } else {
+        const float dr = (float)(rho[i] - 1.0), u[3] = {(float)ux[i], (float)uy[i], (float)uz[i]};
+        float dphi[3][3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const float v = u[d], v2 = v * v;
+            dphi[d][0] = 0.5f * (v2 - v);
+            dphi[d][1] = -v2;
+            dphi[d][2] = 0.5f * (v2 + v);
+        }
+        S* buf = static_cast<S*>(b.buf);
+#pragma unroll
+        for (int s = 0; s < 27; ++s) {
+            const int ix = s % 3, iy = (s / 3) % 3, iz = s / 9;
+            const float A = (float)w1(ix), B = (float)w1(iy), C = (float)w1(iz);
+            const float a = dphi[0][ix], bb = dphi[1][iy], c = dphi[2][iz];
+            const float dprod = a * (B + bb) * (C + c) + A * (bb * (C + c) + B * c);
+            Store<S>::st(buf + (size_t)s * b.stride + cell, dr * ((A + a) * (B + bb) * (C + c)) + dprod);
+        }
+    }
+}
+
+// FP32 storage: cells c0 + 2i and c0 + 2i + 1 in the lanes of f2 values (c0 is even, so the two
+// entries of a slot are one 8-byte store).
+__global__ void __launch_bounds__(128) k_init_eq_pair(BoxGeom b, const double* rho, const double* ux,
+                                                      const double* uy, const double* uz, unsigned c0, unsigned n)
+{
+    const unsigned i = 2u * (blockIdx.x * blockDim.x + threadIdx.x);
+    if (i >= n) return;
+    const bool two = i + 1 < n;
+    const unsigned j = two ? i + 1 : i, cell = c0 + i;
+    const double r[2] = {rho[i], rho[j]}, u[2] = {ux[i], ux[j]}, v[2] = {uy[i], uy[j]}, w[2] = {uz[i], uz[j]};
+    bool plain = true;
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        plain = plain && eq_ordinary(r[k]) && eq_ordinary(u[k]) && eq_ordinary(v[k]) && eq_ordinary(w[k]);
+    if (!plain) {
+        init_cell_fp64<float>(b, cell, r[0], u[0], v[0], w[0]);
+        if (two) init_cell_fp64<float>(b, cell + 1, r[1], u[1], v[1], w[1]);
+        return;
+    }
+    const Dual<f2> dr = dual_of(r[0] - 1.0, r[1] - 1.0);
+    const EqAxis<f2> X = eq_axis(dual_of(u[0], u[1])), Y = eq_axis(dual_of(v[0], v[1])),
+                     Z = eq_axis(dual_of(w[0], w[1]));
+    const Dual<f2> w6 = dual_const<f2>(1.0 / 6.0), w36 = dual_const<f2>(1.0 / 36.0);
+    Dual<f2> P[3];  // dr (A + a) + a
+#pragma unroll
+    for (int ix = 0; ix < 3; ++ix) P[ix] = dual_add(dual_mul(dr, X.f[ix]), X.d[ix]);
+    float* buf = static_cast<float*>(b.buf) + cell;
+#pragma unroll
+    for (int iz = 0; iz < 3; ++iz)
+#pragma unroll
+        for (int iy = 0; iy < 3; ++iy) {
+            const Dual<f2> G = dual_mul(Y.f[iy], Z.f[iz]);
+            // T = [b (C + c) + B c] / 6: A times the bracket is T or 4 T
+            Dual<f2> Bc = dual_mul(w36, Z.d[iz]);
+            if (iy == 1) Bc = dual_scale(Bc, 4.f);
+            const Dual<f2> T = dual_add(dual_mul(w6, dual_mul(Y.d[iy], Z.f[iz])), Bc);
+#pragma unroll
+            for (int ix = 0; ix < 3; ++ix) {
+                const f2 g = dual_sum(dual_mul(P[ix], G), ix == 1 ? dual_scale(T, 4.f) : T);
+                float* p = buf + (size_t)(ix + 3 * iy + 9 * iz) * b.stride;
+                if (two) *reinterpret_cast<float2*>(p) = g.v;
+                else *p = g.v.x;
+            }
+        }
+}
+
 // Density and half-force velocity (Step 7) of every cell, in fp64.  For fp32
 // and 16-bit storage the 27 deviations are summed in fp32 with compensation
 // (sum2_add), which gives the fp64 sums in all but the last bits at fp32 cost,
-// and the three divisions by rho become one reciprocal: the fp64 form below
-// made the kernel fp64-bound on this GPU.  FP64 storage keeps the fp64 form.
+// the three divisions by rho become one reciprocal, the conversions run on the
+// integer pipe (widen) and a force of zero is not added: the fp64 pipe
+// (field_math.cuh) bounds the kernel with every operation it is given, 0.75 ms for 256^3 cells before and 0.52 ms now (bf16: 0.75 and 0.51).
+// FP64 storage keeps the fp64 form.  has_force: any of the force is not zero.
 template <typename S>
-__global__ void k_moments(BoxGeom b, int parity, double Fx, double Fy, double Fz, double* rho, double* ux,
+__global__ void k_moments(BoxGeom b, int parity, int has_force, double Fx, double Fy, double Fz, double* rho, double* ux,
                           double* uy, double* uz, unsigned c0, unsigned n)
 {
     const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -145,11 +178,17 @@ __global__ void k_moments(BoxGeom b, int parity, double Fx, double Fy, double Fz
             if (ey != 0) sum2_add(ys, yc, ey > 0 ? g[s] : -g[s]);
             if (ez != 0) sum2_add(zs, zc, ez > 0 ? g[s] : -g[s]);
         }
-        const double r = 1.0 + ((double)ds + (double)dc), inv = 1.0 / r;
+        const double r = 1.0 + (widen(ds) + widen(dc)), inv = 1.0 / r;
+        double mx = widen(xs) + widen(xc), my = widen(ys) + widen(yc), mz = widen(zs) + widen(zc);
+        if (has_force) {
+            mx += 0.5 * Fx;
+            my += 0.5 * Fy;
+            mz += 0.5 * Fz;
+        }
         if (rho) rho[i] = r;
-        if (ux) ux[i] = ((double)xs + (double)xc + 0.5 * Fx) * inv;
-        if (uy) uy[i] = ((double)ys + (double)yc + 0.5 * Fy) * inv;
-        if (uz) uz[i] = ((double)zs + (double)zc + 0.5 * Fz) * inv;
+        if (ux) ux[i] = mx * inv;
+        if (uy) uy[i] = my * inv;
+        if (uz) uz[i] = mz * inv;
         return;
     }
     double g[27];
@@ -291,7 +330,17 @@ cudaError_t launch_init_eq(int precision, const BoxGeom& b, const double* rho, c
                            const double* uz, unsigned c0, unsigned n, cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
-    FPC_DISPATCH(precision, (k_init_eq<S><<<blocks_for(n, 256), 256, 0, st>>>(b, rho, ux, uy, uz, c0, n)));
+    if (precision == P_FP32) {  // chunks start at even cells, slot rows at 128 bytes
+        if (c0 & 1u) return cudaErrorInvalidValue;
+        k_init_eq_pair<<<blocks_for(n - n / 2, 128), 128, 0, st>>>(b, rho, ux, uy, uz, c0, n);
+        return cudaGetLastError();
+    }
+    switch (precision) {
+        case P_FP64: k_init_eq<double><<<blocks_for(n, 256), 256, 0, st>>>(b, rho, ux, uy, uz, c0, n); break;
+        case P_FP16: k_init_eq<__half><<<blocks_for(n, 256), 256, 0, st>>>(b, rho, ux, uy, uz, c0, n); break;
+        case P_BF16: k_init_eq<__nv_bfloat16><<<blocks_for(n, 256), 256, 0, st>>>(b, rho, ux, uy, uz, c0, n); break;
+        default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 
@@ -299,8 +348,9 @@ cudaError_t launch_moments(int precision, const BoxGeom& b, int parity, double F
                            double* ux, double* uy, double* uz, unsigned c0, unsigned n, cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
-    FPC_DISPATCH(precision,
-                 (k_moments<S><<<blocks_for(n, 256), 256, 0, st>>>(b, parity, Fx, Fy, Fz, rho, ux, uy, uz, c0, n)));
+    const int force = Fx != 0.0 || Fy != 0.0 || Fz != 0.0;
+    FPC_DISPATCH(precision, (k_moments<S><<<blocks_for(n, 256), 256, 0, st>>>(b, parity, force, Fx, Fy, Fz, rho, ux, uy,
+                                                                              uz, c0, n)));
     return cudaGetLastError();
 }
 

@@ -26,7 +26,9 @@
 #include <vector>
 
 #include "rtalloc.h"
+#include "aux.cuh"
 #include "collide.cuh"
+#include "field_math.cuh"
 #include "fpclbm.h"
 #include "hostmem.h"
 #include "internal.h"
@@ -196,37 +198,42 @@ __global__ void __launch_bounds__(256) k_step2d(const Args2<R> a)
     }
 }
 
-// Deviations at the current time whatever the AA parity (as aux.cuh in 3D).
-template <typename S>
-__device__ void load2(const void* bufv, unsigned stride, int nx, int ny, int box, int parity, unsigned cell,
-                      double g[9])
+// Deviations at the current time whatever the AA parity (as aux.cuh in 3D), as T: fp64, or fp32
+// (exact for fp32 and 16-bit storage).
+template <typename S, typename T>
+__device__ __forceinline__ void load2(const void* bufv, unsigned stride, int nx, int ny, int box, int parity,
+                                      unsigned cell, T (&g)[9])
 {
     const S* buf = static_cast<const S*>(bufv);
     if (parity == 0) {
-        for (int s = 0; s < 9; ++s) g[s] = Store<S>::ldd(buf + (size_t)s * stride + cell);
+#pragma unroll
+        for (int s = 0; s < 9; ++s) g[s] = load_as<T>(buf + (size_t)s * stride + cell);
         return;
     }
     const int y = (int)(cell / (unsigned)nx), x = (int)(cell - (unsigned)y * nx);
+#pragma unroll
     for (int s = 0; s < 9; ++s) {
         const int ex = s % 3 - 1, ey = s / 3 - 1;
-        if (box && (x - ex < 0 || x - ex >= nx || y - ey < 0 || y - ey >= ny)) {  // bounce-back
-            g[s] = Store<S>::ldd(buf + (size_t)s * stride + cell);
+        const int sx = x - ex, sy = y - ey;
+        if (box && (sx < 0 || sx >= nx || sy < 0 || sy >= ny)) {  // bounce-back
+            g[s] = load_as<T>(buf + (size_t)s * stride + cell);
             continue;
         }
-        const int sx = (x - ex + nx) % nx, sy = (y - ey + ny) % ny;
-        g[s] = Store<S>::ldd(buf + (size_t)(8 - s) * stride + (size_t)sx + (size_t)nx * sy);
+        const int wx = sx < 0 ? nx - 1 : sx >= nx ? 0 : sx, wy = sy < 0 ? ny - 1 : sy >= ny ? 0 : sy;
+        g[s] = load_as<T>(buf + (size_t)(8 - s) * stride + (size_t)wx + (size_t)nx * wy);
     }
 }
 
 // Product-form equilibrium deviation (equal to C(u)^-1 kappa^eq with the
-// Maxwellian central moments (1, 0, cs^2) per axis, times rho).
+// Maxwellian central moments (1, 0, cs^2) per axis, times rho).  FP32 and 16-bit storage form
+//   g = [dr (A + a) + a] (B + b) + A b
+// on numbers that are sums of two fp32 values (field_math.cuh), rounded to fp32: the fp64 form was
+// bound by the fp64 pipe, 1.92 ms for 4096^2 cells in fp32 against 0.20 ms now; k_moments2d 1.67 ms against 0.53 ms.
+// FP64 storage, and cells out of those numbers' range, take the fp64 form.
 template <typename S>
-__global__ void k_init2d(void* bufv, unsigned stride, unsigned n, const double* rho, const double* ux,
-                         const double* uy)
+__device__ __forceinline__ void init2d_cell_fp64(S* buf, unsigned stride, unsigned c, double r, double u0, double u1)
 {
-    const unsigned c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n) return;
-    const double r = rho[c], u[2] = {ux[c], uy[c]};
+    const double u[2] = {u0, u1};
     double dphi[2][3];
     for (int d = 0; d < 2; ++d) {
         const double v = u[d], v2 = v * v;
@@ -234,7 +241,6 @@ __global__ void k_init2d(void* bufv, unsigned stride, unsigned n, const double* 
         dphi[d][1] = -v2;
         dphi[d][2] = 0.5 * (v2 + v);
     }
-    S* buf = static_cast<S*>(bufv);
     for (int s = 0; s < 9; ++s) {
         const int ix = s % 3, iy = s / 3;
         const double A = w1d(ix), B = w1d(iy), a = dphi[0][ix], b = dphi[1][iy];
@@ -244,11 +250,62 @@ __global__ void k_init2d(void* bufv, unsigned stride, unsigned n, const double* 
 }
 
 template <typename S>
-__global__ void k_moments2d(const void* buf, unsigned stride, int nx, int ny, int box, unsigned n, int parity,
-                            double Fx, double Fy, double* rho, double* ux, double* uy)
+__global__ void k_init2d(void* bufv, unsigned stride, unsigned n, const double* rho, const double* ux,
+                         const double* uy)
 {
     const unsigned c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= n) return;
+    S* buf = static_cast<S*>(bufv);
+    const double r = rho[c], u[2] = {ux[c], uy[c]};
+    if constexpr (!std::is_same<S, double>::value) {
+        if (eq_ordinary(r) && eq_ordinary(u[0]) && eq_ordinary(u[1])) {
+            const Dual<float> dr = dual_of(r - 1.0);
+            const EqAxis<float> X = eq_axis(dual_of(u[0])), Y = eq_axis(dual_of(u[1]));
+            const Dual<float> w6 = dual_const<float>(1.0 / 6.0);
+#pragma unroll
+            for (int ix = 0; ix < 3; ++ix) {
+                const Dual<float> P = dual_add(dual_mul(dr, X.f[ix]), X.d[ix]);
+#pragma unroll
+                for (int iy = 0; iy < 3; ++iy) {
+                    const Dual<float> b = dual_mul(w6, Y.d[iy]);  // A b is this or four times it
+                    Store<S>::st(buf + (size_t)(ix + 3 * iy) * stride + c,
+                                 dual_sum(dual_mul(P, Y.f[iy]), ix == 1 ? dual_scale(b, 4.f) : b));
+                }
+            }
+            return;
+        }
+    }
+    init2d_cell_fp64<S>(buf, stride, c, r, u[0], u[1]);
+}
+
+template <typename S>
+__global__ void k_moments2d(const void* buf, unsigned stride, int nx, int ny, int box, unsigned n, int parity,
+                            int has_force, double Fx, double Fy, double* rho, double* ux, double* uy)
+{
+    const unsigned c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= n) return;
+    if constexpr (!std::is_same<S, double>::value) {
+        float g[9];
+        load2<S>(buf, stride, nx, ny, box, parity, c, g);
+        Sum3 d, x, y;
+#pragma unroll
+        for (int s = 0; s < 9; ++s) {
+            d.add(g[s]);
+            if (s % 3 != 1) x.add(s % 3 == 2 ? g[s] : -g[s]);
+            if (s / 3 != 1) y.add(s / 3 == 2 ? g[s] : -g[s]);
+        }
+        const double r = 1.0 + d.value(), inv = 1.0 / r;
+        // j / r from the reciprocal, with one correction by the quotient's remainder
+        auto over = [&](double j, double F) {
+            if (has_force) j += 0.5 * F;
+            const double q = j * inv;
+            return fma(fma(-q, r, j), inv, q);
+        };
+        if (rho) rho[c] = r;
+        if (ux) ux[c] = over(x.value(), Fx);
+        if (uy) uy[c] = over(y.value(), Fy);
+        return;
+    }
     double g[9];
     load2<S>(buf, stride, nx, ny, box, parity, c, g);
     double dr = 0, jx = 0, jy = 0;
@@ -646,12 +703,12 @@ int fpclbm2d_moments(fpclbm2d_t h, double* rho, double* ux, double* uy, int on_d
         for (int k = 0; k < 3; ++k) o[k] = o[k] ? d + k * n : nullptr;
     }
     const unsigned blocks = (h->ncells + 255) / 256;
-    const int parity = (int)(h->steps & 1);
+    const int parity = (int)(h->steps & 1), force = h->F[0] != 0.0 || h->F[1] != 0.0;
     switch (h->precision) {
-        case FPCLBM_FP64: k_moments2d<double><<<blocks, 256, 0, h->stream>>>(h->d_pop, h->stride, h->nx, h->ny, h->bc == FPCLBM_BC_BOX, h->ncells, parity, h->F[0], h->F[1], o[0], o[1], o[2]); break;
-        case FPCLBM_FP32: k_moments2d<float><<<blocks, 256, 0, h->stream>>>(h->d_pop, h->stride, h->nx, h->ny, h->bc == FPCLBM_BC_BOX, h->ncells, parity, h->F[0], h->F[1], o[0], o[1], o[2]); break;
-        case FPCLBM_FP32_STORE_FP16: k_moments2d<__half><<<blocks, 256, 0, h->stream>>>(h->d_pop, h->stride, h->nx, h->ny, h->bc == FPCLBM_BC_BOX, h->ncells, parity, h->F[0], h->F[1], o[0], o[1], o[2]); break;
-        default: k_moments2d<__nv_bfloat16><<<blocks, 256, 0, h->stream>>>(h->d_pop, h->stride, h->nx, h->ny, h->bc == FPCLBM_BC_BOX, h->ncells, parity, h->F[0], h->F[1], o[0], o[1], o[2]); break;
+        case FPCLBM_FP64: k_moments2d<double><<<blocks, 256, 0, h->stream>>>(h->d_pop, h->stride, h->nx, h->ny, h->bc == FPCLBM_BC_BOX, h->ncells, parity, force, h->F[0], h->F[1], o[0], o[1], o[2]); break;
+        case FPCLBM_FP32: k_moments2d<float><<<blocks, 256, 0, h->stream>>>(h->d_pop, h->stride, h->nx, h->ny, h->bc == FPCLBM_BC_BOX, h->ncells, parity, force, h->F[0], h->F[1], o[0], o[1], o[2]); break;
+        case FPCLBM_FP32_STORE_FP16: k_moments2d<__half><<<blocks, 256, 0, h->stream>>>(h->d_pop, h->stride, h->nx, h->ny, h->bc == FPCLBM_BC_BOX, h->ncells, parity, force, h->F[0], h->F[1], o[0], o[1], o[2]); break;
+        default: k_moments2d<__nv_bfloat16><<<blocks, 256, 0, h->stream>>>(h->d_pop, h->stride, h->nx, h->ny, h->bc == FPCLBM_BC_BOX, h->ncells, parity, force, h->F[0], h->F[1], o[0], o[1], o[2]); break;
     }
     cudaError_t e = cudaGetLastError();
     double* host[3] = {rho, ux, uy};
