@@ -160,8 +160,8 @@ __device__ __forceinline__ void lid_correct_pair(f2 (&g)[27], const CellGeom& G,
 // mode); it reads a valid cell but writes nothing.
 template <typename S, typename R, bool ODD, int BC, bool FORCE, int MODE>
 __device__ __forceinline__ void update_cell(S* __restrict__ buf, const CellGeom& G, unsigned cell,
-                                            const Rates<R>& rt, R Fx, R Fy, R Fz, R om4, R om5, R om6, R om8,
-                                            R om9, const float* closure, int* flag, bool active = true,
+                                            const Rates<R>& rt, R Fx, R Fy, R Fz, const Shear<R>& sh,
+                                            const float* closure, int* flag, bool active = true,
                                             R lid6x = R(0), R lid6z = R(0), const R* smag = nullptr)
 {
     const unsigned stride = G.stride;
@@ -173,7 +173,7 @@ __device__ __forceinline__ void update_cell(S* __restrict__ buf, const CellGeom&
 
     R c2 = R(0);  // Smagorinsky: (C_s Delta D(y))^2 of this cell's row
     if (MODE == MODE_SMAG) c2 = smag[fdiv(cell - fdiv(cell, G.div_nxny) * (unsigned)(G.nx * G.ny), G.div_nx)];
-    const bool ok = collide_cell<R, FORCE, MODE>(g, rt, Fx, Fy, Fz, om4, om5, om6, om8, om9, closure, c2);
+    const bool ok = collide_cell<R, FORCE, MODE>(g, rt, Fx, Fy, Fz, sh, closure, c2);
     if (!ok && active) atomicOr(flag, 1);
 
     // rebuild the store addresses (and the odd step's neighbour table) instead of keeping
@@ -198,8 +198,8 @@ __device__ __forceinline__ void update_cell(S* __restrict__ buf, const CellGeom&
 // correction is applied per lane.
 template <typename S, bool ODD, int BC, bool FORCE, int MODE>
 __device__ __forceinline__ void update_pair(S* __restrict__ buf, const CellGeom& G, unsigned c1, unsigned half,
-                                            unsigned ncells, const Rates<f2>& rt, f2 Fx, f2 Fy, f2 Fz, f2 om4,
-                                            f2 om5, f2 om6, f2 om8, f2 om9, int* flag, f2 lid6x = f2(0.0),
+                                            unsigned ncells, const Rates<f2>& rt, f2 Fx, f2 Fy, f2 Fz,
+                                            const Shear<f2>& sh, int* flag, f2 lid6x = f2(0.0),
                                             f2 lid6z = f2(0.0), const float* closure = nullptr, bool active = true)
 {
     const unsigned stride = G.stride;
@@ -214,7 +214,7 @@ __device__ __forceinline__ void update_pair(S* __restrict__ buf, const CellGeom&
 #pragma unroll
         for (int s = 0; s < 27; ++s) g[s].v.y = Store<S>::ld(load_ptr<S, ODD, BC>(buf, s, n, stride, c2));
     }
-    const bool ok = collide_cell<f2, FORCE, MODE>(g, rt, Fx, Fy, Fz, om4, om5, om6, om8, om9, closure);
+    const bool ok = collide_cell<f2, FORCE, MODE>(g, rt, Fx, Fy, Fz, sh, closure);
     if (!active) return;  // a tail lane of the warp-collective learned mode: nothing to write
     if (!ok) atomicOr(flag, 1);
     asm volatile("" : "+r"(c1));  // rebuild the store addresses (see update_cell)
@@ -269,8 +269,8 @@ struct Store2<__nv_bfloat16> {
 // own addresses), so the odd step keeps its own pairing.
 template <typename S, int BC, bool FORCE, int MODE>
 __device__ __forceinline__ void update_pair_even(S* __restrict__ buf, const CellGeom& G, unsigned t, unsigned ncells,
-                                                 const Rates<f2>& rt, f2 Fx, f2 Fy, f2 Fz, f2 om4, f2 om5, f2 om6,
-                                                 f2 om8, f2 om9, int* flag, f2 lid6x = f2(0.0), f2 lid6z = f2(0.0),
+                                                 const Rates<f2>& rt, f2 Fx, f2 Fy, f2 Fz,
+                                                 const Shear<f2>& sh, int* flag, f2 lid6x = f2(0.0), f2 lid6z = f2(0.0),
                                                  const float* closure = nullptr, bool active = true)
 {
     const unsigned stride = G.stride;
@@ -287,7 +287,7 @@ __device__ __forceinline__ void update_pair_even(S* __restrict__ buf, const Cell
             g[s] = f2(v, v);
         }
     }
-    const bool ok = collide_cell<f2, FORCE, MODE>(g, rt, Fx, Fy, Fz, om4, om5, om6, om8, om9, closure);
+    const bool ok = collide_cell<f2, FORCE, MODE>(g, rt, Fx, Fy, Fz, sh, closure);
     if (!active) return;
     if (!ok) atomicOr(flag, 1);
     asm volatile("" : "+r"(c));  // rebuild the store addresses (see update_cell)
@@ -314,8 +314,8 @@ __device__ __forceinline__ void update_pair_even(S* __restrict__ buf, const Cell
 // address is formed from its own test.  Not for the half channel.
 template <typename S, int BC, bool FORCE, int MODE>
 __device__ __forceinline__ void update_pair_odd_adj(S* __restrict__ buf, const CellGeom& G, unsigned t,
-                                                    const Rates<f2>& rt, f2 Fx, f2 Fy, f2 Fz, f2 om4, f2 om5,
-                                                    f2 om6, f2 om8, f2 om9, int* flag, f2 lid6x = f2(0.0),
+                                                    const Rates<f2>& rt, f2 Fx, f2 Fy, f2 Fz,
+                                                    const Shear<f2>& sh, int* flag, f2 lid6x = f2(0.0),
                                                     f2 lid6z = f2(0.0), const float* closure = nullptr,
                                                     bool active = true)
 {
@@ -349,7 +349,7 @@ __device__ __forceinline__ void update_pair_odd_adj(S* __restrict__ buf, const C
             }
         }
     }
-    const bool ok = collide_cell<f2, FORCE, MODE>(g, rt, Fx, Fy, Fz, om4, om5, om6, om8, om9, closure);
+    const bool ok = collide_cell<f2, FORCE, MODE>(g, rt, Fx, Fy, Fz, sh, closure);
     if (!active) return;
     if (!ok) atomicOr(flag, 1);
     asm volatile("" : "+r"(c));  // rebuild the store addresses (see update_cell)

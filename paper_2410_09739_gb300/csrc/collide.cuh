@@ -42,6 +42,8 @@ namespace fpc {
 template <typename R>
 __device__ __forceinline__ R fmaR(R a, R b, R c) { return fma(a, b, c); }
 template <typename R>
+__device__ __forceinline__ R recipR(R a) { return R(1) / a; }
+template <typename R>
 __device__ __forceinline__ R fminR(R a, R b) { return fmin(a, b); }
 template <typename R>
 __device__ __forceinline__ R fmaxR(R a, R b) { return fmax(a, b); }
@@ -75,44 +77,62 @@ __device__ __forceinline__ void inv3(R& k0, R& k1, R& k2, R u, R u2, R tu, R K)
     k2 = hi;
 }
 
-// inv3 for a line some of whose inputs are known to be zero (Z0, Z1, Z2 for
-// k0, k1, k2): the terms they would feed are left out.  Used in the unit-rate
-// modes, where the moments of orders 3 and 5 are exactly zero after the
-// collision.  A line with K0 && Z0 && Z1 && Z2 does not occur.
-template <typename R, bool K0, bool Z0, bool Z1, bool Z2>
-__device__ __forceinline__ void inv3z(R& k0, R& k1, R& k2, R u, R u2, R tu, R K)
+// Inverse of fwd3 for moments scaled by 1/2 per axis with a non-zero exponent
+// (exact: powers of two), so that the two halvings of a line cost nothing:
+// with M1' = M1 / 2, M2' = M2 / 2 the line is (M2' - M1', k0 - 2 M2', M2' + M1'),
+// seven operations against inv3's eight.  h = u/2, q = u/4, tu = 2u, h2 = u^2/2
+// (read when Z1 only); M2' = tu (q U + k1') + k2'.  Z0, Z1, Z2: k0, k1', k2' known
+// to be zero, their terms left out.  K0: the rest constant K vanishes.
+template <typename R, bool K0, bool Z0 = false, bool Z1 = false, bool Z2 = false>
+__device__ __forceinline__ void inv3h(R& k0, R& k1, R& k2, R h, R q, R tu, R h2, R K)
 {
     constexpr bool UZ = K0 && Z0;  // U = K + k0 vanishes
+    static_assert(!(UZ && Z1 && Z2), "a line of zeros");
     R U = R(0);
     if constexpr (!UZ) {
         if constexpr (K0) U = k0;
         else if constexpr (Z0) U = K;
         else U = K + k0;
     }
-    R M1;
-    if constexpr (UZ) M1 = k1;
-    else if constexpr (Z1) M1 = u * U;
-    else M1 = fmaR(u, U, k1);
-    R M2;
-    if constexpr (Z1 && Z2) {
-        M2 = u2 * U;
+    R M1, M2;
+    if constexpr (Z1) {
+        static_assert(!UZ, "covered by Z0 lines with k1 only");
+        M1 = h * U;
+        if constexpr (Z2) M2 = h2 * U;
+        else M2 = fmaR(h2, U, k2);
     } else {
-        R t;
-        if constexpr (Z1) t = k2;
-        else if constexpr (Z2) t = tu * k1;
-        else t = fmaR(tu, k1, k2);
-        if constexpr (UZ) M2 = t;
-        else M2 = fmaR(u2, U, t);
+        R w = k1;
+        if constexpr (!UZ) w = fmaR(q, U, k1);
+        if constexpr (UZ) M1 = k1;
+        else M1 = fmaR(h, U, k1);
+        if constexpr (Z2) M2 = tu * w;
+        else M2 = fmaR(tu, w, k2);
     }
-    const R h2 = R(0.5) * M2;
-    const R lo = fmaR(R(-0.5), M1, h2);
-    const R hi = fmaR(R(0.5), M1, h2);
     R mid;
-    if constexpr (Z0) mid = -M2;
-    else mid = k0 - M2;
+    if constexpr (Z0) mid = R(-2) * M2;
+    else mid = fmaR(R(-2), M2, k0);
+    const R lo = M2 - M1, hi = M2 + M1;
     k0 = lo;
     k1 = mid;
     k2 = hi;
+}
+
+// What the shear rates leave: 1 - omega_4, 5, 6, 8, 9 of the cell (Step 3), for the unit-rate
+// collision without force scaled like Rates::unit.  own_shear: those of the box's rates.
+template <typename R>
+struct Shear {
+    R k4, k5, k6, k8, k9;
+};
+
+// Unit rates of orders 3-6 and no force: only the moments of orders 0-2 are read (collide_unit).
+__host__ __device__ constexpr bool unit_collision(bool force, int mode) { return r1_mode(mode) && !force; }
+__host__ __device__ constexpr bool scaled_shear(bool force, int mode) { return unit_collision(force, mode) && !learned_mode(mode); }
+
+template <bool FORCE, int MODE, typename R>
+__device__ __forceinline__ Shear<R> own_shear(const Rates<R>& rt)
+{
+    if constexpr (scaled_shear(FORCE, MODE)) return {rt.unit[0], rt.unit[1], rt.unit[2], rt.unit[3], rt.unit[4]};
+    else return {rt.keep[4], rt.keep[5], rt.keep[6], rt.keep[8], rt.keep[9]};
 }
 
 // Rest constants of the three passes (axis z first, then y, then x).
@@ -150,17 +170,200 @@ __device__ __forceinline__ void inv3z(R& k0, R& k1, R& k2, R u, R u2, R tu, R K)
 template <typename R>
 __device__ R closure_delta_omega(const uint32_t* P, const R in[9]);
 
-// Collide one cell in place.  rt: rates of Step 3; Fx, Fy, Fz: body force;
-// om4..om9: the five shear rates (110, 101, 011, 2d1, 2d2), given separately
-// because ensembles carry one shear rate per box; closure: MLP weights
-// (learned mode only); c2 = (C_s Delta D)^2 of the cell (Smagorinsky mode
-// only).  Returns false when rho <= 0 or not finite.
+// The unit-rate collision without force.  kappa~ = kappa^Mv for orders 3-6, and
+// the third- and fifth-order attractors vanish, so the step reads only the moments
+// of orders 0-2 and writes 1 + 3 + 6 + 6 + 1 of them:
+//   forward   raw moments of orders 0-2 from sums over the lines (69 additions),
+//             kappa_ij = m_ij - u_i j_j with one fma each, where the central-moment
+//             transform of all three passes took about 160 operations;
+//   back      scaled lines (inv3h): every moment is formed divided by 2 per axis
+//             with a non-zero exponent, through scaled constants.
+// In all about 340 operations per cell against 430 for the transform-based form
+// (the fp32 kernels issue them packed, two cells at a time; fp64 is bound by them:
+// 32^3 33 -> 27 us a step; bf16 storage, row-staged at 256^3: 0.340 -> 0.311 ms a step).
+//
+// Momentum.  The back transform of an axis gives sum (u U_l + k_l) over its lines,
+// U_l = K + k0_l rounded: the first-order moment must be the residual sum (j_l - u U_l)
+// of those very U_l, each term formed by one fma on the line's own j_l, for the momentum
+// to come back to the last bit.  j - rho u instead (two operations for 5 + 17) repeats an
+// error of u 2^-25 every step of a slowly varying flow: 1.8e-5 of the velocity scale after
+// 1,000 fp32 steps of the 256^3 Taylor-Green vortex, against 5.1e-7 with the residuals.
+// So the planes are transformed back one after the other, and the U_l of a plane give
+// the residual that the next one starts from.
+template <typename R, int MODE>
+__device__ __forceinline__ bool collide_unit(R (&g)[27], const Rates<R>& rt, const Shear<R>& sh, const float* closure)
+{
+    // z lines: S = sum, D = difference, and the sum of all ez^2 terms
+    R S[9], D[9], E[3], m002, m000, m100, m010, m001, m200, m020, m110, m101, m011;
+    {
+        R P[9];
+#pragma unroll
+        for (int l = 0; l < 9; ++l) {
+            const R lo = g[l], mid = g[l + 9], hi = g[l + 18];
+            P[l] = lo + hi;
+            D[l] = hi - lo;
+            S[l] = P[l] + mid;
+        }
+        m002 = ((P[0] + P[1] + P[2]) + (P[3] + P[4] + P[5])) + (P[6] + P[7] + P[8]);
+    }
+    {
+        R s[3], d[3], p[3];
+#pragma unroll
+        for (int y = 0; y < 3; ++y) {
+            p[y] = S[3 * y] + S[3 * y + 2];
+            d[y] = S[3 * y + 2] - S[3 * y];
+            s[y] = p[y] + S[3 * y + 1];
+        }
+        m020 = s[0] + s[2];
+        m000 = m020 + s[1];
+        m200 = (p[0] + p[2]) + p[1];
+        m100 = (d[0] + d[2]) + d[1];
+#pragma unroll
+        for (int x = 0; x < 3; ++x) E[x] = S[x + 6] - S[x];  // y momentum of the columns
+        m010 = (E[0] + E[2]) + E[1];
+        m110 = E[2] - E[0];
+    }
+    {
+        R s[3], d[3];
+#pragma unroll
+        for (int y = 0; y < 3; ++y) {
+            s[y] = (D[3 * y] + D[3 * y + 2]) + D[3 * y + 1];
+            d[y] = D[3 * y + 2] - D[3 * y];
+        }
+        m001 = (s[0] + s[2]) + s[1];
+        m011 = s[2] - s[0];
+        m101 = (d[0] + d[2]) + d[1];
+    }
+    const R drho = m000, rho = R(1) + drho;
+    const bool ok = (rho > R(0)) && (rho < R(1e30));
+    const R inv = recipR(rho);
+    // minus the velocity (each of the transforms below subtracts)
+    const R ninv = -inv;
+    const R nx = m100 * ninv, ny = m010 * ninv, nz = m001 * ninv;
+    // central moments of order 2 (deviations from cs^2 on the diagonal)
+    const R d200 = fmaR(nx, m100, m200), d020 = fmaR(ny, m010, m020), d002 = fmaR(nz, m001, m002);
+    const R d110 = fmaR(nx, m010, m110), d101 = fmaR(nx, m001, m101), d011 = fmaR(ny, m001, m011);
+
+    Shear<R> k = sh;
+    if constexpr (learned_mode(MODE)) {
+        const R third = R(1.0 / 3.0);
+        R in[9];
+        in[0] = d200 - third * drho;  // kappa_200 - cs^2 rho
+        in[1] = d020 - third * drho;
+        in[2] = d002 - third * drho;
+        in[3] = d110;
+        in[4] = d101;
+        in[5] = d011;
+        in[6] = -nx;
+        in[7] = -ny;
+        in[8] = -nz;
+        // the correction only lowers the rates, to 0.02 at least (see collide_cell)
+        const R dw = fminR(closure_delta_omega<R>(reinterpret_cast<const uint32_t*>(closure), in), R(0)), hi = R(0.98);
+        k.k4 = R(0.25) * fminR(sh.k4 - dw, hi);
+        k.k5 = R(0.25) * fminR(sh.k5 - dw, hi);
+        k.k6 = R(0.25) * fminR(sh.k6 - dw, hi);
+        k.k8 = R(1.0 / 6.0) * fminR(sh.k8 - dw, hi);
+        k.k9 = R(1.0 / 6.0) * fminR(sh.k9 - dw, hi);
+    }
+
+    // order 2: a, b, c = kappa~_200, 020, 002 (deviations) / 2; o1, o2, o3 = kappa~_110, 101, 011 / 4;
+    // t = their trace / 6
+    const R o1 = k.k4 * d110, o2 = k.k5 * d101, o3 = k.k6 * d011;
+    const R t = fmaR(rt.unit[5], drho, rt.unit[6] * ((d200 + d020) + d002));
+    const R t1 = k.k8 * (d200 - d020), t2 = k.k9 * (d200 - d002);
+    const R a = (t + t1) + t2, b = fmaR(R(-2), t1, t) + t2, c = fmaR(R(-2), t2, t) + t1;
+    FPC_D(0, 0, 0) = drho;
+    FPC_D(2, 0, 0) = a;
+    FPC_D(0, 2, 0) = b;
+    FPC_D(0, 0, 2) = c;
+    FPC_D(1, 1, 0) = o1;
+    FPC_D(1, 0, 1) = o2;
+    FPC_D(0, 1, 1) = o3;
+    // orders 4 and 6: the attractors, kappa~_220 / 4, kappa~_211 / 8, kappa~_222 / 8
+    if constexpr (eq_mode(MODE)) {
+        FPC_D(2, 2, 0) = FPC_D(2, 0, 2) = FPC_D(0, 2, 2) = R(1.0 / 36.0) * drho;
+        FPC_D(2, 1, 1) = FPC_D(1, 2, 1) = FPC_D(1, 1, 2) = R(0);
+        FPC_D(2, 2, 2) = R(1.0 / 216.0) * drho;
+    } else {
+        const R sixth = R(1.0 / 6.0), nd = R(-1.0 / 36.0) * drho, hinv = R(0.5) * inv;
+        const R ka = sixth + a, kb = sixth + b, kc = sixth + c;  // full kappa~_200 / 2
+        const R ea = fmaR(sixth, a, nd), eb = fmaR(sixth, b, nd);
+        const R p1 = R(8) * o1, p2 = R(8) * o2, p3 = R(8) * o3;
+        const R x220 = fmaR(p1, o1, fmaR(b, ka, ea)) * inv;
+        const R x202 = fmaR(p2, o2, fmaR(c, ka, ea)) * inv;
+        const R x022 = fmaR(p3, o3, fmaR(c, kb, eb)) * inv;
+        const R x211 = fmaR(ka + ka, o3, p1 * o2) * hinv;
+        const R x121 = fmaR(kb + kb, o2, p1 * o3) * hinv;
+        const R x112 = fmaR(kc + kc, o1, p2 * o3) * hinv;
+        R s = fmaR(R(0.5), nd, R(1.0 / 12.0) * t);
+        s = fmaR(ka, x022, fmaR(kb, x202, fmaR(kc, x220, s)));
+        s = fmaR(R(2), fmaR(p1, x112, fmaR(p2, x121, p3 * x211)), s);
+        FPC_D(2, 2, 0) = x220;
+        FPC_D(2, 0, 2) = x202;
+        FPC_D(0, 2, 2) = x022;
+        FPC_D(2, 1, 1) = x211;
+        FPC_D(1, 2, 1) = x121;
+        FPC_D(1, 1, 2) = x112;
+        FPC_D(2, 2, 2) = s * (R(1.0 / 3.0) * inv);
+    }
+
+    // back: plane by plane in p, x lines (moments of total order 3 and 5 are zero) then y lines; the
+    // first-order moments, halved like the others, are the residuals described above
+    const R zero = R(0);
+    {
+        const R hx = R(-0.5) * nx, qx = R(-0.25) * nx, tx = R(-2) * nx, h2x = qx * tx;
+        const R hy = R(-0.5) * ny, qy = R(-0.25) * ny, ty = R(-2) * ny;
+#define FPC_INVX(n, p, Z0, Z1, Z2)                                                                               \
+    inv3h<R, r1(n) * r1(p) == 0.0, Z0, Z1, Z2>(g[3 * (n) + 9 * (p)], g[1 + 3 * (n) + 9 * (p)],                    \
+                                               g[2 + 3 * (n) + 9 * (p)], hx, qx, tx, h2x,                        \
+                                               R(r1(n) * r1(p) * ((n) ? 0.5 : 1.0) * ((p) ? 0.5 : 1.0)))
+        FPC_D(1, 0, 0) = R(0.5) * fmaR(nx, rho, m100);
+        FPC_INVX(0, 0, false, false, false);
+        FPC_INVX(2, 0, false, true, false);
+        {
+            R r[3];
+#pragma unroll
+            for (int x = 0; x < 3; ++x) r[x] = fmaR(ny, R(w1(x)) + g[x], E[x]);
+            FPC_D(0, 1, 0) = R(0.5) * ((r[0] + r[2]) + r[1]);
+        }
+        FPC_INVX(1, 0, false, false, true);
+#pragma unroll
+        for (int x = 0; x < 3; ++x) inv3h<R, false>(g[x], g[x + 3], g[x + 6], hy, qy, ty, zero, R(w1(x)));
+        {
+            R r[9];
+#pragma unroll
+            for (int l = 0; l < 9; ++l) r[l] = fmaR(nz, R(w1(l % 3) * w1(l / 3)) + g[l], D[l]);
+            FPC_D(0, 0, 1) = R(0.5) * (((r[0] + r[2]) + (r[6] + r[8])) + ((r[1] + r[7]) + (r[3] + r[5])) + r[4]);
+        }
+        FPC_INVX(0, 1, false, false, true);
+        FPC_INVX(1, 1, false, true, false);
+        FPC_INVX(2, 1, true, false, true);
+#pragma unroll
+        for (int x = 0; x < 3; ++x) inv3h<R, true>(g[x + 9], g[x + 12], g[x + 15], hy, qy, ty, zero, zero);
+        FPC_INVX(0, 2, false, true, false);
+        FPC_INVX(1, 2, true, false, true);
+        FPC_INVX(2, 2, false, true, false);
+#pragma unroll
+        for (int x = 0; x < 3; ++x)
+            inv3h<R, false>(g[x + 18], g[x + 21], g[x + 24], hy, qy, ty, zero, R(w1(x) * (0.5 / 3.0)));
+#undef FPC_INVX
+    }
+    {
+        const R h = R(-0.5) * nz, q = R(-0.25) * nz, tu = R(-2) * nz;
+#pragma unroll
+        for (int l = 0; l < 9; ++l)
+            inv3h<R, false>(g[l], g[l + 9], g[l + 18], h, q, tu, zero, R(w1(l % 3) * w1(l / 3)));
+    }
+    return ok;
+}
+
+// Any rates, any force: the central-moment transform of all 27 moments.
 template <typename R, bool FORCE, int MODE>
-__device__ __forceinline__ bool collide_cell(R (&g)[27], const Rates<R>& rt, R Fx, R Fy, R Fz, R om4, R om5, R om6,
-                                             R om8, R om9, const float* closure, R c2 = R(0))
+__device__ __forceinline__ bool collide_general(R (&g)[27], const Rates<R>& rt, R Fx, R Fy, R Fz, const Shear<R>& sh,
+                                                const float* closure, R c2)
 {
     constexpr bool R1 = r1_mode(MODE);
-    constexpr bool ODD0 = R1 && !FORCE;  // moments of orders 3 and 5 exactly zero after the collision
+    R k4 = sh.k4, k5 = sh.k5, k6 = sh.k6, k8 = sh.k8, k9 = sh.k9;
     // ---- Step 7 and the first pass (z lines), sharing the line sums ----
     R S[9], Dz[9], Pz[9];
 #pragma unroll
@@ -175,7 +378,7 @@ __device__ __forceinline__ bool collide_cell(R (&g)[27], const Rates<R>& rt, R F
     const R jy = ((S[6] - S[0]) + (S[7] - S[1])) + (S[8] - S[2]);
     const R jz = ((Dz[0] + Dz[1] + Dz[2]) + (Dz[3] + Dz[4] + Dz[5])) + (Dz[6] + Dz[7] + Dz[8]);
     const R rho = R(1) + drho;
-    const R inv_rho = R(1) / rho;
+    const R inv_rho = recipR(rho);
     const bool ok = (rho > R(0)) && (rho < R(1e30));
     R ux, uy, uz;
     if (FORCE) {
@@ -226,12 +429,12 @@ __device__ __forceinline__ bool collide_cell(R (&g)[27], const Rates<R>& rt, R F
         // the correction adds an eddy viscosity nu_t >= 0 (the training label's definition), so it
         // only lowers the rates: omega + min(delta omega, 0), kept above 0.02
         const R dw = fminR(closure_delta_omega<R>(reinterpret_cast<const uint32_t*>(closure), in), R(0));
-        const R lo = R(0.02);
-        om4 = fmaxR(om4 + dw, lo);
-        om5 = fmaxR(om5 + dw, lo);
-        om6 = fmaxR(om6 + dw, lo);
-        om8 = fmaxR(om8 + dw, lo);
-        om9 = fmaxR(om9 + dw, lo);
+        const R hi = R(0.98);
+        k4 = fminR(k4 - dw, hi);
+        k5 = fminR(k5 - dw, hi);
+        k6 = fminR(k6 - dw, hi);
+        k8 = fminR(k8 - dw, hi);
+        k9 = fminR(k9 - dw, hi);
     }
 
     // Smagorinsky eddy viscosity (Sec. 4, turbulent channel LES): nu_t = c2 |S|, the strain rate
@@ -246,10 +449,9 @@ __device__ __forceinline__ bool collide_cell(R (&g)[27], const Rates<R>& rt, R F
         const R o1 = FPC_D(1, 1, 0), o2 = FPC_D(1, 0, 1), o3 = FPC_D(0, 1, 1);
         const R pp = fmaR(q0, q0, fmaR(q1, q1, q2 * q2)) + R(2) * fmaR(o1, o1, fmaR(o2, o2, o3 * o3));
         const R Pn = sqrt(R(2) * pp);
-        const R tau0 = R(1) / om4;
+        const R tau0 = R(1) / rt.om[4];
         const R te = R(0.5) * (tau0 + sqrt(fmaR(tau0, tau0, R(18) * c2 * Pn * inv_rho)));
-        const R w = R(1) / te;
-        om4 = om5 = om6 = om8 = om9 = w;
+        k4 = k5 = k6 = k8 = k9 = R(1) - R(1) / te;
     }
 
     // order 1 (attractor 0, source F).  In exact arithmetic kappa_100 = -F_x/2 and
@@ -280,16 +482,16 @@ __device__ __forceinline__ bool collide_cell(R (&g)[27], const Rates<R>& rt, R F
 
     // order 2: off-diagonal (attractor 0, no source), 2s1 (attractor 3 cs^2 rho),
     // 2d1, 2d2 (attractor 0)
-    FPC_D(1, 1, 0) = (R(1) - om4) * FPC_D(1, 1, 0);
-    FPC_D(1, 0, 1) = (R(1) - om5) * FPC_D(1, 0, 1);
-    FPC_D(0, 1, 1) = (R(1) - om6) * FPC_D(0, 1, 1);
+    FPC_D(1, 1, 0) = k4 * FPC_D(1, 1, 0);
+    FPC_D(1, 0, 1) = k5 * FPC_D(1, 0, 1);
+    FPC_D(0, 1, 1) = k6 * FPC_D(0, 1, 1);
     {
         const R d200 = FPC_D(2, 0, 0), d020 = FPC_D(0, 2, 0), d002 = FPC_D(0, 0, 2);
         const R y2s = (d200 + d020) + d002;
         const R y2d1 = d200 - d020, y2d2 = d200 - d002;
         const R t2s = fmaR(rt.om[7], drho, rt.keep[7] * y2s);  // attractor deviation: drho
-        const R t2d1 = (R(1) - om8) * y2d1;
-        const R t2d2 = (R(1) - om9) * y2d2;
+        const R t2d1 = k8 * y2d1;
+        const R t2d2 = k9 * y2d2;
         FPC_D(2, 0, 0) = third * ((t2s + t2d1) + t2d2);
         FPC_D(0, 2, 0) = third * (fmaR(R(-2), t2d1, t2s) + t2d2);
         FPC_D(0, 0, 2) = third * (fmaR(R(-2), t2d2, t2s) + t2d1);
@@ -307,11 +509,7 @@ __device__ __forceinline__ bool collide_cell(R (&g)[27], const Rates<R>& rt, R F
     }
 
     // order 3 (attractors 0): pairs (120,102), (210,012), (201,021), and 111
-    if constexpr (ODD0) {
-        FPC_D(1, 2, 0) = FPC_D(1, 0, 2) = FPC_D(2, 1, 0) = R(0);
-        FPC_D(0, 1, 2) = FPC_D(2, 0, 1) = FPC_D(0, 2, 1) = R(0);
-        FPC_D(1, 1, 1) = R(0);
-    } else if constexpr (R1) {  // with force: half the sources
+    if constexpr (R1) {  // half the sources
         FPC_D(1, 2, 0) = R(0.5) * s120;
         FPC_D(1, 0, 2) = R(0.5) * s102;
         FPC_D(2, 1, 0) = R(0.5) * s210;
@@ -368,21 +566,12 @@ __device__ __forceinline__ bool collide_cell(R (&g)[27], const Rates<R>& rt, R F
             A112 = fmaR(third + pc, o110, R(2) * o011 * o101) * inv_rho;
         }
         if constexpr (R1) {
-            if constexpr (FORCE) {
-                FPC_D(2, 2, 0) = fmaR(R(0.5), s220, A220);
-                FPC_D(2, 0, 2) = fmaR(R(0.5), s202, A202);
-                FPC_D(0, 2, 2) = fmaR(R(0.5), s022, A022);
-                FPC_D(2, 1, 1) = fmaR(R(0.5), s211, A211);
-                FPC_D(1, 2, 1) = fmaR(R(0.5), s121, A121);
-                FPC_D(1, 1, 2) = fmaR(R(0.5), s112, A112);
-            } else {
-                FPC_D(2, 2, 0) = A220;
-                FPC_D(2, 0, 2) = A202;
-                FPC_D(0, 2, 2) = A022;
-                FPC_D(2, 1, 1) = A211;
-                FPC_D(1, 2, 1) = A121;
-                FPC_D(1, 1, 2) = A112;
-            }
+            FPC_D(2, 2, 0) = fmaR(R(0.5), s220, A220);
+            FPC_D(2, 0, 2) = fmaR(R(0.5), s202, A202);
+            FPC_D(0, 2, 2) = fmaR(R(0.5), s022, A022);
+            FPC_D(2, 1, 1) = fmaR(R(0.5), s211, A211);
+            FPC_D(1, 2, 1) = fmaR(R(0.5), s121, A121);
+            FPC_D(1, 1, 2) = fmaR(R(0.5), s112, A112);
         } else {
         const R d220 = FPC_D(2, 2, 0), d202 = FPC_D(2, 0, 2), d022 = FPC_D(0, 2, 2);
         const R y4s = (d220 + d202) + d022, y4d1 = (d220 + d202) - d022, y4d2 = d220 - d202;
@@ -417,9 +606,7 @@ __device__ __forceinline__ bool collide_cell(R (&g)[27], const Rates<R>& rt, R F
     if (FORCE) s222 = R(2) * ((fx * FPC_D(1, 2, 2) + fy * FPC_D(2, 1, 2)) + fz * FPC_D(2, 2, 1));
 
     // order 5: attractors from post-collision second and third moments
-    if constexpr (ODD0) {
-        FPC_D(1, 2, 2) = FPC_D(2, 1, 2) = FPC_D(2, 2, 1) = R(0);
-    } else {
+    {
         R A122 = R(0), A212 = R(0), A221 = R(0);
         if constexpr (!eq_mode(MODE)) {
             const R K200 = third + pa, K020 = third + pb, K002 = third + pc;
@@ -432,7 +619,7 @@ __device__ __forceinline__ bool collide_cell(R (&g)[27], const Rates<R>& rt, R F
             A221 = c * (fmaR(K200, FPC_D(0, 2, 1), K020 * FPC_D(2, 0, 1)) +
                         fmaR(R(4) * o110, k111, R(2) * fmaR(o011, FPC_D(2, 1, 0), o101 * FPC_D(1, 2, 0))));
         }
-        if constexpr (R1) {  // with force (ODD0 handled above)
+        if constexpr (R1) {
             FPC_D(1, 2, 2) = fmaR(R(0.5), s122, A122);
             FPC_D(2, 1, 2) = fmaR(R(0.5), s212, A212);
             FPC_D(2, 2, 1) = fmaR(R(0.5), s221, A221);
@@ -464,7 +651,7 @@ __device__ __forceinline__ bool collide_cell(R (&g)[27], const Rates<R>& rt, R F
             A222 = (t - ninth * drho) * (third * inv_rho);
         }
         if constexpr (R1) {
-            FPC_D(2, 2, 2) = FORCE ? fmaR(R(0.5), s222, A222) : A222;
+            FPC_D(2, 2, 2) = fmaR(R(0.5), s222, A222);
         } else {
             R t222 = fmaR(rt.om[26], A222, rt.keep[26] * FPC_D(2, 2, 2));
             if (FORCE) t222 = fmaR(rt.src[26], s222, t222);
@@ -473,24 +660,7 @@ __device__ __forceinline__ bool collide_cell(R (&g)[27], const Rates<R>& rt, R F
     }
 
     // ---- Steps 4+5: back to populations (passes in reverse order) ----
-    if constexpr (ODD0) {
-        // x lines at fixed (n, p); inputs of total order 3 or 5 are zero
-#define FPC_INVC(n, p, Z0, Z1, Z2)                                                                        \
-    inv3z<R, r1(n) * r1(p) == 0.0, Z0, Z1, Z2>(g[3 * (n) + 9 * (p)], g[1 + 3 * (n) + 9 * (p)],           \
-                                               g[2 + 3 * (n) + 9 * (p)], ux, ux2, tux, R(r1(n) * r1(p)))
-        FPC_INVC(0, 0, false, false, false);
-        FPC_INVC(1, 0, false, false, true);
-        FPC_INVC(2, 0, false, true, false);
-        FPC_INVC(0, 1, false, false, true);
-        FPC_INVC(1, 1, false, true, false);
-        FPC_INVC(2, 1, true, false, true);
-        FPC_INVC(0, 2, false, true, false);
-        FPC_INVC(1, 2, true, false, true);
-        FPC_INVC(2, 2, false, true, false);
-#undef FPC_INVC
-    } else {
-        FPC_PASS_C(inv3)
-    }
+    FPC_PASS_C(inv3)
     FPC_PASS_B(inv3)
 #pragma unroll
     for (int l = 0; l < 9; ++l) {
@@ -498,6 +668,18 @@ __device__ __forceinline__ bool collide_cell(R (&g)[27], const Rates<R>& rt, R F
         inv3<R, false>(g[l], g[l + 9], g[l + 18], uz, uz2, tuz, R(Kd));
     }
     return ok;
+}
+
+// Collide one cell in place.  rt: rates of Step 3; Fx, Fy, Fz: body force;
+// sh: 1 minus the five shear rates (110, 101, 011, 2d1, 2d2; own_shear, or
+// an ensemble box's); closure: MLP weights (learned mode only); c2 = (C_s Delta D)^2 of the cell (Smagorinsky mode
+// only).  Returns false when rho <= 0 or not finite.
+template <typename R, bool FORCE, int MODE>
+__device__ __forceinline__ bool collide_cell(R (&g)[27], const Rates<R>& rt, R Fx, R Fy, R Fz, const Shear<R>& sh,
+                                             const float* closure, R c2 = R(0))
+{
+    if constexpr (unit_collision(FORCE, MODE)) return collide_unit<R, MODE>(g, rt, sh, closure);
+    else return collide_general<R, FORCE, MODE>(g, rt, Fx, Fy, Fz, sh, closure, c2);
 }
 
 #undef FPC_PASS_B

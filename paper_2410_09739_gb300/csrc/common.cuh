@@ -70,12 +70,36 @@ __device__ __forceinline__ unsigned fdiv(unsigned n, const FastDiv& f)
 // numbering of Appendix D Step 3 (0:000 ... 26:222).  Entries 0..3 (the
 // conserved moments) are not read by the kernels: they cancel in exact
 // arithmetic (see collide.cuh, order 1).
+// unit: the five shear keeps 1 - omega_4, 5, 6 over 4 and 1 - omega_8, 9 over 6, and omega_7 and
+// 1 - omega_7 over 6: the factors of the unit-rate collision, whose moments are scaled for the back
+// transform (collide.cuh).
 template <typename R>
 struct Rates {
     R om[27];
     R keep[27];
     R src[27];
+    R unit[7];
 };
+
+// The rates of one box in arithmetic type R, from omega_0..26 in fp64.
+template <typename R>
+inline Rates<R> make_rates(const double om[27])
+{
+    Rates<R> r;
+    for (int j = 0; j < 27; ++j) {
+        r.om[j] = R(om[j]);
+        r.keep[j] = R(1.0 - om[j]);
+        r.src[j] = R(1.0 - 0.5 * om[j]);
+    }
+    r.unit[0] = R((1.0 - om[4]) / 4);
+    r.unit[1] = R((1.0 - om[5]) / 4);
+    r.unit[2] = R((1.0 - om[6]) / 4);
+    r.unit[3] = R((1.0 - om[8]) / 6);
+    r.unit[4] = R((1.0 - om[9]) / 6);
+    r.unit[5] = R(om[7] / 6);
+    r.unit[6] = R((1.0 - om[7]) / 6);
+    return r;
+}
 
 // Arguments of one single-box step launch.
 template <typename R>

@@ -8,6 +8,7 @@
 // tile list; each tile runs the same per-cell update as a single box, with
 // the box's own geometry and shear rate 1/tau_b.  Boxes never exchange data.
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "rtalloc.h"
@@ -15,6 +16,27 @@
 #include "handle.h"
 
 namespace fpc {
+
+template <typename R>
+__device__ __forceinline__ R both(float v)
+{
+    if constexpr (std::is_same<R, f2>::value) return f2(v, v);
+    else return v;
+}
+
+// One shear rate for all five of a box (the same values as Rates::keep and Rates::unit of a single
+// box with that rate, so both advance a box bit for bit alike).
+template <bool FORCE, int MODE, typename R>
+__device__ __forceinline__ Shear<R> box_shear(const EnsBox& B)
+{
+    if constexpr (scaled_shear(FORCE, MODE)) {
+        const R k4 = both<R>(__ldg(&B.keep4)), k6 = both<R>(__ldg(&B.keep6));
+        return {k4, k4, k4, k6, k6};
+    } else {
+        const R k = both<R>(__ldg(&B.keep));
+        return {k, k, k, k, k};
+    }
+}
 
 template <bool ODD, bool FORCE, int MODE, int MINB>
 __global__ void __launch_bounds__(256, MINB) k_ens_step(const EnsArgs a)
@@ -36,13 +58,13 @@ __global__ void __launch_bounds__(256, MINB) k_ens_step(const EnsArgs a)
         G.div_nxny.d = __ldg(&B.div_nxny.d);
         G.div_nxny.m = __ldg(&B.div_nxny.m);
         G.div_nxny.s = __ldg(&B.div_nxny.s);
-        const float om = __ldg(&B.om_shear);
+        const Shear<float> sh = box_shear<FORCE, MODE, float>(B);
         float* buf = base + __ldg(&B.off);
         for (unsigned c = threadIdx.x; c < a.tile_cells; c += blockDim.x) {
             const unsigned cell = first + c;
             if (cell >= ncells) break;
-            update_cell<float, float, ODD, BC_PERIODIC, FORCE, MODE>(buf, G, cell, a.rates, a.Fx, a.Fy, a.Fz, om, om, om, om,
-                                                               om, nullptr, a.flag);
+            update_cell<float, float, ODD, BC_PERIODIC, FORCE, MODE>(buf, G, cell, a.rates, a.Fx, a.Fy, a.Fz,
+                                                               sh, nullptr, a.flag);
         }
     }
 }
@@ -72,23 +94,22 @@ __global__ void __launch_bounds__(128, MINB) k_ens_pair(const EnsArgs a)
         G.div_nxny.d = __ldg(&B.div_nxny.d);
         G.div_nxny.m = __ldg(&B.div_nxny.m);
         G.div_nxny.s = __ldg(&B.div_nxny.s);
-        const float om = __ldg(&B.om_shear);
-        const f2 om2(om, om);
+        const Shear<f2> sh = box_shear<FORCE, MODE, f2>(B);
         float* buf = base + __ldg(&B.off);
         for (unsigned c = threadIdx.x; c < half; c += blockDim.x) {
             if (ODD && (G.nx & 1) == 0) {  // even nx: neighbouring cells, shared neighbour table
                 if (first + 2 * c >= ncells) break;
                 update_pair_odd_adj<float, BC_PERIODIC, FORCE, MODE>(buf, G, first / 2 + c, a.rates2, a.Fx2, a.Fy2,
-                                                                     a.Fz2, om2, om2, om2, om2, om2, a.flag);
+                                                                     a.Fz2, sh, a.flag);
             } else if (ODD) {
                 const unsigned c1 = first + c;
                 if (c1 >= ncells) break;
                 update_pair<float, ODD, BC_PERIODIC, FORCE, MODE>(buf, G, c1, half, ncells, a.rates2, a.Fx2, a.Fy2,
-                                                                  a.Fz2, om2, om2, om2, om2, om2, a.flag);
+                                                                  a.Fz2, sh, a.flag);
             } else {  // neighbouring cells first + 2c, first + 2c + 1 (tiles and box blocks are even-aligned)
                 if (first + 2 * c >= ncells) break;
                 update_pair_even<float, BC_PERIODIC, FORCE, MODE>(buf, G, first / 2 + c, ncells, a.rates2, a.Fx2,
-                                                                  a.Fy2, a.Fz2, om2, om2, om2, om2, om2, a.flag);
+                                                                  a.Fy2, a.Fz2, sh, a.flag);
             }
         }
     }
@@ -283,7 +304,10 @@ extern "C" int fpclbm_create_ensemble(fpclbm_t* out, int n_boxes, const int* dim
                 E.nz = bx.nz;
                 E.div_nx = make_fastdiv((unsigned)bx.nx);
                 E.div_nxny = make_fastdiv((unsigned)(bx.nx * bx.ny));
-                E.om_shear = (float)(1.0 / bx.tau);
+                const double keep = 1.0 - 1.0 / bx.tau;
+                E.keep = (float)keep;
+                E.keep4 = (float)(keep / 4);
+                E.keep6 = (float)(keep / 6);
                 E.tile0 = bx.tile0;
                 for (unsigned t = 0; t < bx.ntiles; ++t) tb[bx.tile0 + t] = (unsigned)b;
             }

@@ -173,11 +173,7 @@ StepArgs<R> make_args(const fpclbm* h)
     a.Fz = (R)h->F[2];
     a.lid6x = (R)(6.0 * h->lid[0]);
     a.lid6z = (R)(6.0 * h->lid[1]);
-    for (int j = 0; j < 27; ++j) {
-        a.rates.om[j] = (R)h->omega[j];
-        a.rates.keep[j] = (R)(1.0 - h->omega[j]);
-        a.rates.src[j] = (R)(1.0 - 0.5 * h->omega[j]);
-    }
+    a.rates = make_rates<R>(h->omega);
     a.flag = h->d_flag;
     a.closure = h->d_closure;
     a.smag = h->diffusion == FPCLBM_DIFF_FP_SMAGORINSKY ? static_cast<const R*>(h->d_smag) : nullptr;
@@ -192,19 +188,11 @@ EnsArgs make_ens_args(const fpclbm* h)
     a.tile_box = h->d_tile_box;
     a.ntiles = h->ntiles;
     a.tile_cells = (unsigned)h->tile_cells;
-    for (int j = 0; j < 27; ++j) {
-        a.rates.om[j] = (float)h->omega[j];
-        a.rates.keep[j] = (float)(1.0 - h->omega[j]);
-        a.rates.src[j] = (float)(1.0 - 0.5 * h->omega[j]);
-    }
+    a.rates = make_rates<float>(h->omega);
     a.Fx = (float)h->F[0];
     a.Fy = (float)h->F[1];
     a.Fz = (float)h->F[2];
-    for (int j = 0; j < 27; ++j) {
-        a.rates2.om[j] = f2(a.rates.om[j], a.rates.om[j]);
-        a.rates2.keep[j] = f2(a.rates.keep[j], a.rates.keep[j]);
-        a.rates2.src[j] = f2(a.rates.src[j], a.rates.src[j]);
-    }
+    a.rates2 = make_rates<f2>(h->omega);
     a.Fx2 = f2(a.Fx, a.Fx);
     a.Fy2 = f2(a.Fy, a.Fy);
     a.Fz2 = f2(a.Fz, a.Fz);

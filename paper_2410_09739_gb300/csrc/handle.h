@@ -31,7 +31,7 @@ struct EnsBox {
     unsigned stride, ncells;
     int nx, ny, nz;
     FastDiv div_nx, div_nxny;
-    float om_shear;
+    float keep, keep4, keep6;  // 1 - omega of the box's shear rate, and that over 4 and over 6
     unsigned tile0;
 };
 

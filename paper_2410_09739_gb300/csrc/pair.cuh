@@ -9,8 +9,9 @@
 // contraction choices (a*b+c written with fma on one side and not the other).
 //
 // f2 supplies what collide_cell needs from its arithmetic type R: + - * and
-// unary minus, fmaR, construction from a constant, 1/x, and a comparison that
-// is true only when it holds on both lanes (collide_cell's validity check).
+// unary minus, fmaR, construction from a constant, the reciprocal recipR, and a
+// comparison that is true only when it holds on both lanes (collide_cell's
+// validity check).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -36,6 +37,7 @@ __device__ __forceinline__ bool operator<(f2 a, f2 b) { return a.v.x < b.v.x && 
 // overloads of collide.cuh's fmaR, fminR, fmaxR (a non-template exact match wins for f2)
 __device__ __forceinline__ f2 fminR(f2 a, f2 b) { return f2(fminf(a.v.x, b.v.x), fminf(a.v.y, b.v.y)); }
 __device__ __forceinline__ f2 fmaxR(f2 a, f2 b) { return f2(fmaxf(a.v.x, b.v.x), fmaxf(a.v.y, b.v.y)); }
+__device__ __forceinline__ f2 recipR(f2 a) { return f2(__frcp_rn(a.v.x), __frcp_rn(a.v.y)); }
 __device__ __forceinline__ f2 fmaR(f2 a, f2 b, f2 c) { return f2(__ffma2_rn(a.v, b.v, c.v)); }
 
 }  // namespace fpc

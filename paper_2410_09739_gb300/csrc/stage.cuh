@@ -485,8 +485,8 @@ __global__ void __launch_bounds__(32 * (NCW + 1), stage_min_blocks(NCW, FORCE, M
         mbar_arrive(empty_in + 8u * ki);
         bool fine = true;
         if (act)
-            fine = collide_cell<f2, FORCE, MODE>(g, rt, a.Fx, a.Fy, a.Fz, rt.om[4], rt.om[5], rt.om[6], rt.om[8],
-                                                 rt.om[9], nullptr);
+            fine = collide_cell<f2, FORCE, MODE>(g, rt, a.Fx, a.Fy, a.Fz, own_shear<FORCE, MODE>(rt),
+                                                 nullptr);
         if (!fine) atomicOr(a.flag, 1);
         if (i >= (unsigned)nso && !mbar_wait_or_abort(empty_out + 8u * ko, pout ^ 1u, abort)) return;
         const uint32_t aout = out0 + (unsigned)ko * STB;

@@ -29,8 +29,8 @@ __global__ void __launch_bounds__(256, MINB) k_step(const StepArgs<R> a)
     G.div_nx = a.div_nx;
     G.div_nxny = a.div_nxny;
     const Rates<R>& rt = a.rates;
-    update_cell<S, R, ODD, BC, FORCE, MODE>(static_cast<S*>(a.buf), G, cell, rt, a.Fx, a.Fy, a.Fz, rt.om[4],
-                                            rt.om[5], rt.om[6], rt.om[8], rt.om[9], a.closure, a.flag, active,
+    update_cell<S, R, ODD, BC, FORCE, MODE>(static_cast<S*>(a.buf), G, cell, rt, a.Fx, a.Fy, a.Fz,
+                                            own_shear<FORCE, MODE>(rt), a.closure, a.flag, active,
                                             a.lid6x, a.lid6z, a.smag);
 }
 
@@ -102,8 +102,8 @@ __global__ void __launch_bounds__(128, MINB) k_step_pipe(const StepArgs<R> a, un
             const S* src = sm + (size_t)stage * 27 * T + tid;
 #pragma unroll
             for (int s = 0; s < 27; ++s) g[s] = Store<S>::ld(src + s * T);
-            const bool ok = collide_cell<R, FORCE, MODE>(g, rt, a.Fx, a.Fy, a.Fz, rt.om[4], rt.om[5], rt.om[6],
-                                                         rt.om[8], rt.om[9], a.closure);
+            const bool ok = collide_cell<R, FORCE, MODE>(g, rt, a.Fx, a.Fy, a.Fz, own_shear<FORCE, MODE>(rt),
+                                                         a.closure);
             if (!ok) atomicOr(a.flag, 1);
             Nbr n;
             if (ODD) n = make_nbr<BC>(G, cell);
@@ -167,17 +167,17 @@ __global__ void __launch_bounds__(128, MINB) k_step_pair(const StepArgs<f2> a, u
     G.div_nxny = a.div_nxny;
     const Rates<f2>& rt = a.rates;
     if constexpr (ODD && ADJ)  // neighbouring cells 2 c1, 2 c1 + 1 with a shared neighbour table
-        update_pair_odd_adj<S, BC, FORCE, MODE>(static_cast<S*>(a.buf), G, c1, rt, a.Fx, a.Fy, a.Fz, rt.om[4],
-                                                rt.om[5], rt.om[6], rt.om[8], rt.om[9], a.flag, a.lid6x, a.lid6z,
-                                                a.closure, active);
+        update_pair_odd_adj<S, BC, FORCE, MODE>(static_cast<S*>(a.buf), G, c1, rt, a.Fx, a.Fy, a.Fz,
+                                                own_shear<FORCE, MODE>(rt), a.flag, a.lid6x, a.lid6z, a.closure,
+                                                active);
     else if constexpr (ODD)  // cells c1 and c1 + half
         update_pair<S, ODD, BC, FORCE, MODE>(static_cast<S*>(a.buf), G, c1, half, a.ncells, rt, a.Fx, a.Fy, a.Fz,
-                                             rt.om[4], rt.om[5], rt.om[6], rt.om[8], rt.om[9], a.flag, a.lid6x,
-                                             a.lid6z, a.closure, active);
+                                             own_shear<FORCE, MODE>(rt), a.flag, a.lid6x, a.lid6z, a.closure,
+                                             active);
     else  // neighbouring cells 2 c1 and 2 c1 + 1, vector loads and stores
         update_pair_even<S, BC, FORCE, MODE>(static_cast<S*>(a.buf), G, c1, a.ncells, rt, a.Fx, a.Fy, a.Fz,
-                                             rt.om[4], rt.om[5], rt.om[6], rt.om[8], rt.om[9], a.flag, a.lid6x,
-                                             a.lid6z, a.closure, active);
+                                             own_shear<FORCE, MODE>(rt), a.flag, a.lid6x, a.lid6z, a.closure,
+                                             active);
 }
 
 // The launch arguments with every scalar duplicated into both lanes.
@@ -202,6 +202,7 @@ inline StepArgs<f2> pair_args(const StepArgs<float>& a)
         p.rates.keep[j] = f2(a.rates.keep[j], a.rates.keep[j]);
         p.rates.src[j] = f2(a.rates.src[j], a.rates.src[j]);
     }
+    for (int j = 0; j < 7; ++j) p.rates.unit[j] = f2(a.rates.unit[j], a.rates.unit[j]);
     p.flag = a.flag;
     p.closure = a.closure;
     p.smag = nullptr;
