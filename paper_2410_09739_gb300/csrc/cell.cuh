@@ -158,7 +158,7 @@ __device__ __forceinline__ void lid_correct_pair(f2 (&g)[27], const CellGeom& G,
 
 // active = false: the lane only takes part in warp-collective work (learned
 // mode); it reads a valid cell but writes nothing.
-template <typename S, typename R, bool ODD, int BC, bool FORCE, int MODE>
+template <typename S, typename R, bool ODD, int BC, int FORCE, int MODE>
 __device__ __forceinline__ void update_cell(S* __restrict__ buf, const CellGeom& G, unsigned cell,
                                             const Rates<R>& rt, R Fx, R Fy, R Fz, const Shear<R>& sh,
                                             const float* closure, int* flag, bool active = true,
@@ -196,7 +196,7 @@ __device__ __forceinline__ void update_cell(S* __restrict__ buf, const CellGeom&
 // addresses.  c2 is recomputed after the collision (from the uniform half)
 // rather than kept live through it.  Every boundary kind; the moving-wall
 // correction is applied per lane.
-template <typename S, bool ODD, int BC, bool FORCE, int MODE>
+template <typename S, bool ODD, int BC, int FORCE, int MODE>
 __device__ __forceinline__ void update_pair(S* __restrict__ buf, const CellGeom& G, unsigned c1, unsigned half,
                                             unsigned ncells, const Rates<f2>& rt, f2 Fx, f2 Fy, f2 Fz,
                                             const Shear<f2>& sh, int* flag, f2 lid6x = f2(0.0),
@@ -267,7 +267,7 @@ struct Store2<__nv_bfloat16> {
 // second cell lies past the end (odd cell count) updates c alone.  Which
 // thread updates which cell is free within a step (each cell touches only its
 // own addresses), so the odd step keeps its own pairing.
-template <typename S, int BC, bool FORCE, int MODE>
+template <typename S, int BC, int FORCE, int MODE>
 __device__ __forceinline__ void update_pair_even(S* __restrict__ buf, const CellGeom& G, unsigned t, unsigned ncells,
                                                  const Rates<f2>& rt, f2 Fx, f2 Fy, f2 Fz,
                                                  const Shear<f2>& sh, int* flag, f2 lid6x = f2(0.0), f2 lid6z = f2(0.0),
@@ -312,7 +312,7 @@ __device__ __forceinline__ void update_pair_even(S* __restrict__ buf, const Cell
 // within the cells' own slots (plus 1).  In the closed box the x walls give
 // the two cells different tests for e_x != 0, so there the second cell's
 // address is formed from its own test.  Not for the half channel.
-template <typename S, int BC, bool FORCE, int MODE>
+template <typename S, int BC, int FORCE, int MODE>
 __device__ __forceinline__ void update_pair_odd_adj(S* __restrict__ buf, const CellGeom& G, unsigned t,
                                                     const Rates<f2>& rt, f2 Fx, f2 Fy, f2 Fz,
                                                     const Shear<f2>& sh, int* flag, f2 lid6x = f2(0.0),

@@ -26,6 +26,10 @@ namespace fpc {
 // MODE_LEARNED_R1 is the learned mode with the unit rates of orders 3-6.
 enum { MODE_FP = 0, MODE_EQ = 1, MODE_LEARNED = 2, MODE_SMAG = 3, MODE_FP_R1 = 4, MODE_EQ_R1 = 5, MODE_LEARNED_R1 = 6 };
 
+// Body force of a step kernel: none, any, or along x only (the unit-rate modes have a collision of
+// their own for the last, see collide.cuh).
+enum { FORCE_NONE = 0, FORCE_ANY = 1, FORCE_X = 2 };
+
 // FP or MCM attractors with the full register-cap / pipelined / paired variant set.
 __host__ __device__ constexpr bool plain_mode(int m) { return m == MODE_FP || m == MODE_EQ || m == MODE_FP_R1 || m == MODE_EQ_R1; }
 __host__ __device__ constexpr bool eq_mode(int m) { return m == MODE_EQ || m == MODE_EQ_R1; }

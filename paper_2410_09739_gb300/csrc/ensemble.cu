@@ -26,7 +26,7 @@ __device__ __forceinline__ R both(float v)
 
 // One shear rate for all five of a box (the same values as Rates::keep and Rates::unit of a single
 // box with that rate, so both advance a box bit for bit alike).
-template <bool FORCE, int MODE, typename R>
+template <int FORCE, int MODE, typename R>
 __device__ __forceinline__ Shear<R> box_shear(const EnsBox& B)
 {
     if constexpr (scaled_shear(FORCE, MODE)) {
@@ -38,7 +38,7 @@ __device__ __forceinline__ Shear<R> box_shear(const EnsBox& B)
     }
 }
 
-template <bool ODD, bool FORCE, int MODE, int MINB>
+template <bool ODD, int FORCE, int MODE, int MINB>
 __global__ void __launch_bounds__(256, MINB) k_ens_step(const EnsArgs a)
 {
     float* __restrict__ base = static_cast<float*>(a.buf);
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(256, MINB) k_ens_step(const EnsArgs a)
 // thread (one vector access per slot where the pair's values are adjacent; see
 // update_pair_even and update_pair_odd_adj), except on the odd step of a box
 // with odd nx, where cells t and t + tile/2 do.
-template <bool ODD, bool FORCE, int MODE, int MINB>
+template <bool ODD, int FORCE, int MODE, int MINB>
 __global__ void __launch_bounds__(128, MINB) k_ens_pair(const EnsArgs a)
 {
     float* __restrict__ base = static_cast<float*>(a.buf);
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(128, MINB) k_ens_pair(const EnsArgs a)
 }
 
 // Resident blocks of 128 threads per SM of the even-step paired kernel with a given cap.
-template <bool FORCE, int MODE, int MINB>
+template <int FORCE, int MODE, int MINB>
 static int occ_even_pair()
 {
     static int n = 0;  // benign race: every thread computes the same value
@@ -133,7 +133,7 @@ static int occ_even_pair()
     return n;
 }
 
-template <bool ODD, bool FORCE, int MODE>
+template <bool ODD, int FORCE, int MODE>
 static cudaError_t go(const EnsArgs& a, int block, int minb, int grid, int variant, cudaStream_t st)
 {
     if (variant == 2) {
@@ -163,10 +163,13 @@ template <int MODE>
 static cudaError_t go_mode(int odd, int force, const EnsArgs& a, int block, int minb, int grid, int variant,
                            cudaStream_t st)
 {
-    if (odd) return force ? go<true, true, MODE>(a, block, minb, grid, variant, st)
-                          : go<true, false, MODE>(a, block, minb, grid, variant, st);
-    return force ? go<false, true, MODE>(a, block, minb, grid, variant, st)
-                 : go<false, false, MODE>(a, block, minb, grid, variant, st);
+#define FPC_ENS_GO(O, F) go<O, F, MODE>(a, block, minb, grid, variant, st)
+    if constexpr (r1_mode(MODE)) {
+        if (force == FORCE_X) return odd ? FPC_ENS_GO(true, FORCE_X) : FPC_ENS_GO(false, FORCE_X);
+    }
+    if (odd) return force ? FPC_ENS_GO(true, FORCE_ANY) : FPC_ENS_GO(true, FORCE_NONE);
+    return force ? FPC_ENS_GO(false, FORCE_ANY) : FPC_ENS_GO(false, FORCE_NONE);
+#undef FPC_ENS_GO
 }
 
 cudaError_t launch_ens_step(int odd, int force, int mode, const EnsArgs& a, int block, int minb, int grid,
@@ -189,11 +192,11 @@ static int ens_occupancy(int block, int minb, int variant)
     int n = 0;
     cudaError_t e;
     if (variant == 2)
-        e = minb == 3 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ens_pair<false, false, MODE, 3>, block, 0)
-                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ens_pair<false, false, MODE, 4>, block, 0);
+        e = minb == 3 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ens_pair<false, FORCE_NONE, MODE, 3>, block, 0)
+                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ens_pair<false, FORCE_NONE, MODE, 4>, block, 0);
     else
-        e = minb == 3 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ens_step<false, false, MODE, 3>, block, 0)
-                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ens_step<false, false, MODE, 2>, block, 0);
+        e = minb == 3 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ens_step<false, FORCE_NONE, MODE, 3>, block, 0)
+                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ens_step<false, FORCE_NONE, MODE, 2>, block, 0);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return 1;

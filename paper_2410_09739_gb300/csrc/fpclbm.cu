@@ -215,7 +215,12 @@ BoxGeom geom_of(const fpclbm* h, const Box& b)
     return g;
 }
 
-bool has_force(const fpclbm* h) { return h->F[0] != 0.0 || h->F[1] != 0.0 || h->F[2] != 0.0; }
+// FORCE_* kind of the handle's body force.
+int force_kind(const fpclbm* h)
+{
+    if (h->F[1] != 0.0 || h->F[2] != 0.0) return FORCE_ANY;
+    return h->F[0] != 0.0 ? FORCE_X : FORCE_NONE;
+}
 
 // Collision mode of the step kernel.  A box or ensemble in the FP or MCM mode whose rates of
 // orders 3-6 (Step 3 indices 10..26) are all exactly 1 takes the unit-rate variant, which sets
@@ -276,11 +281,11 @@ int upload_smag(fpclbm* h)
 cudaError_t one_step(fpclbm* h, long long t, cudaStream_t st, int block, int minb, int grid, int pipe)
 {
     if (h->ensemble)
-        return launch_ens_step((int)(t & 1), has_force(h), mode_of(h), make_ens_args(h), block, minb, grid, pipe, st);
+        return launch_ens_step((int)(t & 1), force_kind(h), mode_of(h), make_ens_args(h), block, minb, grid, pipe, st);
     const StepArgs<double> a64 = make_args<double>(h);
     const StepArgs<float> a32 = make_args<float>(h);
     StepLaunch cfg{block, minb, pipe, pipe == 3 ? grid : 2};  // variant 3 keeps its stage count in grid
-    return launch_step(h->precision, (int)(t & 1), kernel_bc(h), has_force(h), mode_of(h), a64, a32, cfg, st);
+    return launch_step(h->precision, (int)(t & 1), kernel_bc(h), force_kind(h), mode_of(h), a64, a32, cfg, st);
 }
 
 void drop_graph(fpclbm* h)
@@ -415,7 +420,7 @@ int stage_threads(const fpclbm* h)
 std::string tune_key(const fpclbm* h)
 {
     char buf[160];
-    std::snprintf(buf, sizeof buf, "dev%d/p%d/bc%d/f%d/m%d/%s/%llu", h->device, h->precision, kernel_bc(h), (int)has_force(h),
+    std::snprintf(buf, sizeof buf, "dev%d/p%d/bc%d/f%d/m%d/%s/%llu", h->device, h->precision, kernel_bc(h), force_kind(h),
                   mode_of(h), h->ensemble ? "ens" : "box", (unsigned long long)(h->total_cells >> 20));
     return buf;
 }

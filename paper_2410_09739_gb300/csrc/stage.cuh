@@ -319,7 +319,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 // Resident blocks per SM the registers are capped for: four blocks of 4 consumer warps (96
 // registers) for the unit-rate collision without force, which fits them without spilling, three
 // for the other modes; two blocks of 6 consumer warps (146 registers); one block of 8.
-__host__ __device__ constexpr int stage_min_blocks(int NCW, bool FORCE, int MODE)
+__host__ __device__ constexpr int stage_min_blocks(int NCW, int FORCE, int MODE)
 {
     return NCW == 4 ? ((r1_mode(MODE) && !FORCE) ? 4 : 3) : NCW == 6 ? 2 : 1;
 }
@@ -328,7 +328,7 @@ __host__ __device__ constexpr int stage_min_blocks(int NCW, bool FORCE, int MODE
 // CB, the bytes of one slot chunk of a stage, is a compile-time constant, so that every
 // shared-memory access of the compute phase is an immediate offset; a tile holds R whole rows,
 // R nx <= CB / sizeof(S).
-template <typename S, bool ODD, int BC, bool FORCE, int MODE, int NCW>
+template <typename S, bool ODD, int BC, int FORCE, int MODE, int NCW>
 __global__ void __launch_bounds__(32 * (NCW + 1), stage_min_blocks(NCW, FORCE, MODE)) k_step_stage(const StepArgs<f2> a, const FastDiv div_tpp,
                                                                const unsigned ntiles, const int R, const int nsi)
 {
@@ -510,7 +510,7 @@ inline int stage_rows(int nx, int ny, int cap)
 }
 
 // Launch: one CTA per resident slot (persistent); nsi input and kStageOut output stages.
-template <typename S, bool ODD, int BC, bool FORCE, int MODE, int NCW>
+template <typename S, bool ODD, int BC, int FORCE, int MODE, int NCW>
 cudaError_t step_go_stage_ncw(const StepArgs<float>& a, int nsi, cudaStream_t st)
 {
     constexpr int TC = 64 * NCW;
@@ -554,7 +554,7 @@ cudaError_t step_go_stage_ncw(const StepArgs<float>& a, int nsi, cudaStream_t st
 
 // Tiles of up to 256 cells (4 consumer warps) for rows of at most 256 cells, of 384 (6 consumer
 // warps, two blocks per SM) for rows of at most 384, else of 512 (8 consumer warps).
-template <typename S, bool ODD, int BC, bool FORCE, int MODE>
+template <typename S, bool ODD, int BC, int FORCE, int MODE>
 cudaError_t step_go_stage(const StepArgs<float>& a, int nsi, cudaStream_t st)
 {
     if ((a.nx * sizeof(S)) % 16 != 0 || a.nx > 512 || a.nx < 2 || nsi < 2 || nsi > 6) return cudaErrorInvalidValue;

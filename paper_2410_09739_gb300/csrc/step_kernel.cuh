@@ -10,7 +10,7 @@
 
 namespace fpc {
 
-template <typename S, typename R, bool ODD, int BC, bool FORCE, int MODE, int MINB>
+template <typename S, typename R, bool ODD, int BC, int FORCE, int MODE, int MINB>
 __global__ void __launch_bounds__(256, MINB) k_step(const StepArgs<R> a)
 {
     unsigned cell = blockIdx.x * blockDim.x + threadIdx.x;
@@ -57,7 +57,7 @@ __device__ __forceinline__ void cp_async_wait()
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
-template <typename S, typename R, bool ODD, int BC, bool FORCE, int MODE, int MINB>
+template <typename S, typename R, bool ODD, int BC, int FORCE, int MODE, int MINB>
 __global__ void __launch_bounds__(128, MINB) k_step_pipe(const StepArgs<R> a, unsigned ntiles)
 {
     static_assert(sizeof(S) == 4 || sizeof(S) == 8, "cp.async moves 4, 8 or 16 bytes");
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(128, MINB) k_step_pipe(const StepArgs<R> a, un
     cp_async_wait<0>();
 }
 
-template <typename S, typename R, bool ODD, int BC, bool FORCE, int MODE, int MINB>
+template <typename S, typename R, bool ODD, int BC, int FORCE, int MODE, int MINB>
 cudaError_t step_go_pipe(const StepArgs<R>& a, cudaStream_t st)
 {
     constexpr int T = 128;
@@ -147,7 +147,7 @@ cudaError_t step_go_pipe(const StepArgs<R>& a, cudaStream_t st)
 // cell still reads and writes only its own AA addresses.
 // ---------------------------------------------------------------------------
 
-template <typename S, bool ODD, int BC, bool FORCE, int MODE, int MINB, bool ADJ>
+template <typename S, bool ODD, int BC, int FORCE, int MODE, int MINB, bool ADJ>
 __global__ void __launch_bounds__(128, MINB) k_step_pair(const StepArgs<f2> a, unsigned half)
 {
     unsigned c1 = blockIdx.x * blockDim.x + threadIdx.x;
@@ -209,7 +209,7 @@ inline StepArgs<f2> pair_args(const StepArgs<float>& a)
     return p;
 }
 
-template <typename S, bool ODD, int BC, bool FORCE, int MODE, int MINB>
+template <typename S, bool ODD, int BC, int FORCE, int MODE, int MINB>
 cudaError_t step_go_pair(const StepArgs<float>& a, cudaStream_t st)
 {
     const unsigned half = (a.ncells + 1) / 2;
@@ -229,7 +229,7 @@ cudaError_t step_go_pair(const StepArgs<float>& a, cudaStream_t st)
     return cudaGetLastError();
 }
 
-template <typename S, typename R, bool ODD, int BC, bool FORCE, int MODE, int MINB>
+template <typename S, typename R, bool ODD, int BC, int FORCE, int MODE, int MINB>
 cudaError_t step_go(const StepArgs<R>& a, const StepLaunch& cfg, cudaStream_t st)
 {
     // paired variant: fp32 arithmetic, FP and MCM modes, every boundary kind, one register cap
@@ -262,7 +262,7 @@ cudaError_t step_go(const StepArgs<R>& a, const StepLaunch& cfg, cudaStream_t st
 // modes (every boundary kind); 1 (no cap) and 2 (128 registers) for the
 // learned mode on boxes with resting walls, whose tensor-core MLP keeps the
 // cell's state live.  fp64 and the Smagorinsky mode have one variant each.
-template <typename S, typename R, bool ODD, int BC, bool FORCE, int MODE>
+template <typename S, typename R, bool ODD, int BC, int FORCE, int MODE>
 cudaError_t step_by_minb(const StepArgs<R>& a, const StepLaunch& cfg, cudaStream_t st)
 {
     constexpr bool fp32_capped = sizeof(R) == 4 && plain_mode(MODE);
@@ -279,25 +279,29 @@ cudaError_t step_by_minb(const StepArgs<R>& a, const StepLaunch& cfg, cudaStream
     }
 }
 
-template <typename S, typename R, bool ODD, int BC, bool FORCE>
+template <typename S, typename R, bool ODD, int BC, int FORCE>
 cudaError_t step_by_mode(int mode, const StepArgs<R>& a, const StepLaunch& cfg, cudaStream_t st)
 {
     switch (mode) {
-        case MODE_FP: return step_by_minb<S, R, ODD, BC, FORCE, MODE_FP>(a, cfg, st);
-        case MODE_EQ: return step_by_minb<S, R, ODD, BC, FORCE, MODE_EQ>(a, cfg, st);
         case MODE_FP_R1: return step_by_minb<S, R, ODD, BC, FORCE, MODE_FP_R1>(a, cfg, st);  // unit rates, orders >= 3
         case MODE_EQ_R1: return step_by_minb<S, R, ODD, BC, FORCE, MODE_EQ_R1>(a, cfg, st);
-        case MODE_LEARNED:  // periodic and channel boxes (the closure's training data come from them)
-            if constexpr (BC == BC_PERIODIC || BC == BC_WALLS_Y)
-                return step_by_minb<S, R, ODD, BC, FORCE, MODE_LEARNED>(a, cfg, st);
-            break;
-        case MODE_LEARNED_R1:  // the same with unit rates of orders 3-6
+        case MODE_LEARNED_R1:  // periodic and channel boxes (the closure's training data come from them)
             if constexpr (BC == BC_PERIODIC || BC == BC_WALLS_Y)
                 return step_by_minb<S, R, ODD, BC, FORCE, MODE_LEARNED_R1>(a, cfg, st);
             break;
-        case MODE_SMAG:  // resting walls
-            if constexpr (bc_fixed(BC)) return step_by_minb<S, R, ODD, BC, FORCE, MODE_SMAG>(a, cfg, st);
-            break;
+    }
+    if constexpr (FORCE != FORCE_X) {
+        switch (mode) {
+            case MODE_FP: return step_by_minb<S, R, ODD, BC, FORCE, MODE_FP>(a, cfg, st);
+            case MODE_EQ: return step_by_minb<S, R, ODD, BC, FORCE, MODE_EQ>(a, cfg, st);
+            case MODE_LEARNED:
+                if constexpr (BC == BC_PERIODIC || BC == BC_WALLS_Y)
+                    return step_by_minb<S, R, ODD, BC, FORCE, MODE_LEARNED>(a, cfg, st);
+                break;
+            case MODE_SMAG:  // resting walls
+                if constexpr (bc_fixed(BC)) return step_by_minb<S, R, ODD, BC, FORCE, MODE_SMAG>(a, cfg, st);
+                break;
+        }
     }
     return cudaErrorInvalidValue;
 }
@@ -305,8 +309,13 @@ cudaError_t step_by_mode(int mode, const StepArgs<R>& a, const StepLaunch& cfg, 
 template <typename S, typename R, bool ODD, int BC>
 cudaError_t step_by_force(int force, int mode, const StepArgs<R>& a, const StepLaunch& cfg, cudaStream_t st)
 {
-    return force ? step_by_mode<S, R, ODD, BC, true>(mode, a, cfg, st)
-                 : step_by_mode<S, R, ODD, BC, false>(mode, a, cfg, st);
+    switch (force) {
+        case FORCE_NONE: return step_by_mode<S, R, ODD, BC, FORCE_NONE>(mode, a, cfg, st);
+        case FORCE_X:  // the unit-rate modes only; the others have no use for the distinction
+            if (r1_mode(mode)) return step_by_mode<S, R, ODD, BC, FORCE_X>(mode, a, cfg, st);
+            break;
+    }
+    return step_by_mode<S, R, ODD, BC, FORCE_ANY>(mode, a, cfg, st);
 }
 
 template <typename S, typename R, bool ODD>
