@@ -133,11 +133,25 @@ __device__ __forceinline__ void lid_correct(R g[27], R lid6x, R lid6z)
     }
 }
 
-// Whether a cell lies in the top row y = ny - 1 (the moving wall's neighbours).
-__device__ __forceinline__ bool top_row(const CellGeom& G, unsigned cell)
+// Row y of a cell.
+__device__ __forceinline__ unsigned row_of(const CellGeom& G, unsigned cell)
 {
-    const unsigned y = fdiv(cell - fdiv(cell, G.div_nxny) * (unsigned)(G.nx * G.ny), G.div_nx);
-    return y + 1 == (unsigned)G.ny;
+    return fdiv(cell - fdiv(cell, G.div_nxny) * (unsigned)(G.nx * G.ny), G.div_nx);
+}
+
+// Whether a cell lies in the top row y = ny - 1 (the moving wall's neighbours).
+__device__ __forceinline__ bool top_row(const CellGeom& G, unsigned cell) { return row_of(G, cell) + 1 == (unsigned)G.ny; }
+
+// (C_s Delta D(y))^2 of the two cells of a pair (Smagorinsky modes).
+template <int MODE>
+__device__ __forceinline__ f2 smag_pair(const CellGeom& G, unsigned ca, unsigned cb, const void* smag)
+{
+    if constexpr (smag_mode(MODE)) {
+        const float* t = static_cast<const float*>(smag);
+        return f2(t[row_of(G, ca)], t[row_of(G, cb)]);
+    } else {
+        return f2(0.f, 0.f);
+    }
 }
 
 // The moving-wall correction for the lanes of a pair whose cell lies in the
@@ -162,7 +176,7 @@ template <typename S, typename R, bool ODD, int BC, int FORCE, int MODE>
 __device__ __forceinline__ void update_cell(S* __restrict__ buf, const CellGeom& G, unsigned cell,
                                             const Rates<R>& rt, R Fx, R Fy, R Fz, const Shear<R>& sh,
                                             const float* closure, int* flag, bool active = true,
-                                            R lid6x = R(0), R lid6z = R(0), const R* smag = nullptr)
+                                            R lid6x = R(0), R lid6z = R(0), const void* smag = nullptr)
 {
     const unsigned stride = G.stride;
     R g[27];
@@ -172,7 +186,7 @@ __device__ __forceinline__ void update_cell(S* __restrict__ buf, const CellGeom&
     for (int s = 0; s < 27; ++s) g[s] = Store<S>::ld(load_ptr<S, ODD, BC>(buf, s, n, stride, cell));
 
     R c2 = R(0);  // Smagorinsky: (C_s Delta D(y))^2 of this cell's row
-    if (MODE == MODE_SMAG) c2 = smag[fdiv(cell - fdiv(cell, G.div_nxny) * (unsigned)(G.nx * G.ny), G.div_nx)];
+    if constexpr (smag_mode(MODE)) c2 = static_cast<const R*>(smag)[row_of(G, cell)];
     const bool ok = collide_cell<R, FORCE, MODE>(g, rt, Fx, Fy, Fz, sh, closure, c2);
     if (!ok && active) atomicOr(flag, 1);
 
@@ -200,7 +214,8 @@ template <typename S, bool ODD, int BC, int FORCE, int MODE>
 __device__ __forceinline__ void update_pair(S* __restrict__ buf, const CellGeom& G, unsigned c1, unsigned half,
                                             unsigned ncells, const Rates<f2>& rt, f2 Fx, f2 Fy, f2 Fz,
                                             const Shear<f2>& sh, int* flag, f2 lid6x = f2(0.0),
-                                            f2 lid6z = f2(0.0), const float* closure = nullptr, bool active = true)
+                                            f2 lid6z = f2(0.0), const float* closure = nullptr, bool active = true,
+                                            const void* smag = nullptr)
 {
     const unsigned stride = G.stride;
     f2 g[27];
@@ -214,7 +229,8 @@ __device__ __forceinline__ void update_pair(S* __restrict__ buf, const CellGeom&
 #pragma unroll
         for (int s = 0; s < 27; ++s) g[s].v.y = Store<S>::ld(load_ptr<S, ODD, BC>(buf, s, n, stride, c2));
     }
-    const bool ok = collide_cell<f2, FORCE, MODE>(g, rt, Fx, Fy, Fz, sh, closure);
+    const bool ok = collide_cell<f2, FORCE, MODE>(g, rt, Fx, Fy, Fz, sh, closure,
+                                                  smag_pair<MODE>(G, c1, c1 + half < ncells ? c1 + half : c1, smag));
     if (!active) return;  // a tail lane of the warp-collective learned mode: nothing to write
     if (!ok) atomicOr(flag, 1);
     asm volatile("" : "+r"(c1));  // rebuild the store addresses (see update_cell)
@@ -271,7 +287,8 @@ template <typename S, int BC, int FORCE, int MODE>
 __device__ __forceinline__ void update_pair_even(S* __restrict__ buf, const CellGeom& G, unsigned t, unsigned ncells,
                                                  const Rates<f2>& rt, f2 Fx, f2 Fy, f2 Fz,
                                                  const Shear<f2>& sh, int* flag, f2 lid6x = f2(0.0), f2 lid6z = f2(0.0),
-                                                 const float* closure = nullptr, bool active = true)
+                                                 const float* closure = nullptr, bool active = true,
+                                                 const void* smag = nullptr)
 {
     const unsigned stride = G.stride;
     unsigned c = 2 * t;
@@ -287,7 +304,8 @@ __device__ __forceinline__ void update_pair_even(S* __restrict__ buf, const Cell
             g[s] = f2(v, v);
         }
     }
-    const bool ok = collide_cell<f2, FORCE, MODE>(g, rt, Fx, Fy, Fz, sh, closure);
+    const bool ok = collide_cell<f2, FORCE, MODE>(g, rt, Fx, Fy, Fz, sh, closure,
+                                                  smag_pair<MODE>(G, c, two ? c + 1 : c, smag));
     if (!active) return;
     if (!ok) atomicOr(flag, 1);
     asm volatile("" : "+r"(c));  // rebuild the store addresses (see update_cell)
@@ -317,10 +335,8 @@ __device__ __forceinline__ void update_pair_odd_adj(S* __restrict__ buf, const C
                                                     const Rates<f2>& rt, f2 Fx, f2 Fy, f2 Fz,
                                                     const Shear<f2>& sh, int* flag, f2 lid6x = f2(0.0),
                                                     f2 lid6z = f2(0.0), const float* closure = nullptr,
-                                                    bool active = true)
+                                                    bool active = true, const void* smag = nullptr)
 {
-    static_assert(BC == BC_PERIODIC || BC == BC_WALLS_Y || BC == BC_WALLS_Y_LID || BC == BC_BOX_LID,
-                  "no symmetry plane");
     const unsigned stride = G.stride;
     unsigned c = 2 * t;
     f2 g[27];
@@ -343,13 +359,15 @@ __device__ __forceinline__ void update_pair_odd_adj(S* __restrict__ buf, const C
                     g[s].v.y = Store<S>::ld(in2 ? buf + (size_t)(26 - s) * stride + ((unsigned)x2 + n.yz[iy][iz])
                                                 : buf + (size_t)s * stride + (c + 1));
                 } else {
-                    const int w = inside<BC>(n, ix, iy, iz) ? (ix == 0 ? wp : wm) : 0;
+                    const bool moves = BC == BC_HALF_CHANNEL ? iy != 2 || n.yin[2] : inside<BC>(n, ix, iy, iz);
+                    const int w = moves ? (ix == 0 ? wp : wm) : 0;
                     g[s].v.y = Store<S>::ld(p + 1 + w);
                 }
             }
         }
     }
-    const bool ok = collide_cell<f2, FORCE, MODE>(g, rt, Fx, Fy, Fz, sh, closure);
+    const bool ok = collide_cell<f2, FORCE, MODE>(g, rt, Fx, Fy, Fz, sh, closure,
+                                                  smag_pair<MODE>(G, c, c + 1, smag));
     if (!active) return;
     if (!ok) atomicOr(flag, 1);
     asm volatile("" : "+r"(c));  // rebuild the store addresses (see update_cell)
@@ -373,7 +391,8 @@ __device__ __forceinline__ void update_pair_odd_adj(S* __restrict__ buf, const C
                                  : buf + (size_t)(26 - s) * stride + (c + 1),
                              g[s].v.y);
             } else {
-                const int w = inside<BC>(n, 2 - ix, 2 - iy, 2 - iz) ? (ix == 2 ? wp : wm) : 0;
+                const bool moves = BC == BC_HALF_CHANNEL ? iy != 0 || n.yin[2] : inside<BC>(n, 2 - ix, 2 - iy, 2 - iz);
+                const int w = moves ? (ix == 2 ? wp : wm) : 0;
                 Store<S>::st(p + 1 + w, g[s].v.y);
             }
         }

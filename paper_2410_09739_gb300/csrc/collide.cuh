@@ -44,6 +44,8 @@ __device__ __forceinline__ R fmaR(R a, R b, R c) { return fma(a, b, c); }
 template <typename R>
 __device__ __forceinline__ R recipR(R a) { return R(1) / a; }
 template <typename R>
+__device__ __forceinline__ R sqrtR(R a) { return sqrt(a); }
+template <typename R>
 __device__ __forceinline__ R fminR(R a, R b) { return fmin(a, b); }
 template <typename R>
 __device__ __forceinline__ R fmaxR(R a, R b) { return fmax(a, b); }
@@ -126,7 +128,7 @@ struct Shear {
 
 // Unit rates of orders 3-6 and no force or one along x: collide_unit.
 __host__ __device__ constexpr bool unit_collision(int force, int mode) { return r1_mode(mode) && force != FORCE_ANY; }
-__host__ __device__ constexpr bool scaled_shear(int force, int mode) { return unit_collision(force, mode) && !learned_mode(mode); }
+__host__ __device__ constexpr bool scaled_shear(int force, int mode) { return unit_collision(force, mode) && !learned_mode(mode) && !smag_mode(mode); }
 
 template <int FORCE, int MODE, typename R>
 __device__ __forceinline__ Shear<R> own_shear(const Rates<R>& rt)
@@ -170,6 +172,24 @@ __device__ __forceinline__ Shear<R> own_shear(const Rates<R>& rt)
 template <typename R>
 __device__ R closure_delta_omega(const uint32_t* P, const R in[9]);
 
+// Smagorinsky eddy viscosity (Sec. 4, turbulent channel LES): nu_t = c2 |S|, the strain rate from
+// the deviatoric non-equilibrium second moments Pi^d (of the central moments' deviations d from the
+// rest state) at the effective time tau, S = -Pi^d / (2 rho cs^2 tau), tau = tau0 + nu_t / cs^2; the
+// positive root of tau^2 - tau0 tau - c2 |Pi^d| / (2 rho cs^4) = 0, whose inverse replaces all five
+// shear rates.
+template <typename R>
+__device__ __forceinline__ R smagorinsky_tau(R d200, R d020, R d002, R d110, R d101, R d011, R drho, R inv_rho, R c2,
+                                             R tau0)
+{
+    const R third = R(1.0 / 3.0);
+    const R p0 = d200 - third * drho, p1 = d020 - third * drho, p2 = d002 - third * drho;
+    const R tr = third * ((p0 + p1) + p2);
+    const R q0 = p0 - tr, q1 = p1 - tr, q2 = p2 - tr;
+    const R pp = fmaR(q0, q0, fmaR(q1, q1, q2 * q2)) + R(2) * fmaR(d110, d110, fmaR(d101, d101, d011 * d011));
+    const R Pn = sqrtR(R(2) * pp);
+    return R(0.5) * (tau0 + sqrtR(fmaR(tau0, tau0, R(18) * c2 * Pn * inv_rho)));
+}
+
 // The unit-rate collision, without force (first) or with a force along x (XF, below).
 // Without force kappa~ = kappa^Mv for orders 3-6, and
 // the third- and fifth-order attractors vanish, so the step reads only the moments
@@ -199,7 +219,7 @@ __device__ R closure_delta_omega(const uint32_t* P, const R in[9]);
 // with the sources of all three components (384x192x192 channel, bf16: 0.426 -> 0.366 ms a step).
 template <typename R, bool XF, int MODE>
 __device__ __forceinline__ bool collide_unit(R (&g)[27], const Rates<R>& rt, R Fx, const Shear<R>& sh,
-                                             const float* closure)
+                                             const float* closure, R c2)
 {
     // z lines: S = sum, D = difference, P the sum of the ez^2 terms
     R S[9], D[9], P[9], E[3], m002, m000, m100, m010, m001, m200, m020, m110, m101, m011;
@@ -331,6 +351,11 @@ __device__ __forceinline__ bool collide_unit(R (&g)[27], const Rates<R>& rt, R F
         k.k6 = R(0.25) * fminR(sh.k6 - dw, hi);
         k.k8 = R(1.0 / 6.0) * fminR(sh.k8 - dw, hi);
         k.k9 = R(1.0 / 6.0) * fminR(sh.k9 - dw, hi);
+    }
+    if constexpr (smag_mode(MODE)) {
+        const R ke = R(1) - recipR(smagorinsky_tau(d200, d020, d002, d110, d101, d011, drho, inv, c2, recipR(rt.om[4])));
+        k.k4 = k.k5 = k.k6 = R(0.25) * ke;
+        k.k8 = k.k9 = R(1.0 / 6.0) * ke;
     }
 
     // order 2: a, b, c = kappa~_200, 020, 002 (deviations) / 2; o1, o2, o3 = kappa~_110, 101, 011 / 4;
@@ -547,20 +572,9 @@ __device__ __forceinline__ bool collide_general(R (&g)[27], const Rates<R>& rt, 
         k9 = fminR(k9 - dw, hi);
     }
 
-    // Smagorinsky eddy viscosity (Sec. 4, turbulent channel LES): nu_t = c2 |S|, the strain rate
-    // from the deviatoric non-equilibrium second moments Pi^d at the effective time tau,
-    // S = -Pi^d / (2 rho cs^2 tau), tau = tau0 + nu_t / cs^2; the positive root of
-    // tau^2 - tau0 tau - c2 |Pi^d| / (2 rho cs^4) = 0 replaces all five shear rates.
     if constexpr (MODE == MODE_SMAG) {
-        const R p0 = FPC_D(2, 0, 0) - third * drho, p1 = FPC_D(0, 2, 0) - third * drho;
-        const R p2 = FPC_D(0, 0, 2) - third * drho;
-        const R tr = third * ((p0 + p1) + p2);
-        const R q0 = p0 - tr, q1 = p1 - tr, q2 = p2 - tr;
-        const R o1 = FPC_D(1, 1, 0), o2 = FPC_D(1, 0, 1), o3 = FPC_D(0, 1, 1);
-        const R pp = fmaR(q0, q0, fmaR(q1, q1, q2 * q2)) + R(2) * fmaR(o1, o1, fmaR(o2, o2, o3 * o3));
-        const R Pn = sqrt(R(2) * pp);
-        const R tau0 = R(1) / rt.om[4];
-        const R te = R(0.5) * (tau0 + sqrt(fmaR(tau0, tau0, R(18) * c2 * Pn * inv_rho)));
+        const R te = smagorinsky_tau(FPC_D(2, 0, 0), FPC_D(0, 2, 0), FPC_D(0, 0, 2), FPC_D(1, 1, 0), FPC_D(1, 0, 1),
+                                     FPC_D(0, 1, 1), drho, inv_rho, c2, R(1) / rt.om[4]);
         k4 = k5 = k6 = k8 = k9 = R(1) - R(1) / te;
     }
 
@@ -782,13 +796,13 @@ __device__ __forceinline__ bool collide_general(R (&g)[27], const Rates<R>& rt, 
 
 // Collide one cell in place.  rt: rates of Step 3; Fx, Fy, Fz: body force;
 // sh: 1 minus the five shear rates (110, 101, 011, 2d1, 2d2; own_shear, or
-// an ensemble box's); closure: MLP weights (learned mode only); c2 = (C_s Delta D)^2 of the cell (Smagorinsky mode
+// an ensemble box's); closure: MLP weights (learned mode only); c2 = (C_s Delta D)^2 of the cell (Smagorinsky modes
 // only).  Returns false when rho <= 0 or not finite.
 template <typename R, int FORCE, int MODE>
 __device__ __forceinline__ bool collide_cell(R (&g)[27], const Rates<R>& rt, R Fx, R Fy, R Fz, const Shear<R>& sh,
                                              const float* closure, R c2 = R(0))
 {
-    if constexpr (unit_collision(FORCE, MODE)) return collide_unit<R, FORCE == FORCE_X, MODE>(g, rt, Fx, sh, closure);
+    if constexpr (unit_collision(FORCE, MODE)) return collide_unit<R, FORCE == FORCE_X, MODE>(g, rt, Fx, sh, closure, c2);
     else return collide_general<R, FORCE, MODE>(g, rt, Fx, Fy, Fz, sh, closure, c2);
 }
 

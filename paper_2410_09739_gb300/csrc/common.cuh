@@ -23,8 +23,10 @@ namespace fpc {
 // then their attractors plus half their sources (kappa + 1 (kappa^Mv - kappa)
 // + (1 - 1/2) sigma), with no grouping; without force the pre-collision
 // moments of those orders are not formed at all.
-// MODE_LEARNED_R1 is the learned mode with the unit rates of orders 3-6.
-enum { MODE_FP = 0, MODE_EQ = 1, MODE_LEARNED = 2, MODE_SMAG = 3, MODE_FP_R1 = 4, MODE_EQ_R1 = 5, MODE_LEARNED_R1 = 6 };
+// MODE_LEARNED_R1 and MODE_SMAG_R1 are the learned and Smagorinsky modes with the unit rates of
+// orders 3-6 (MODE_SMAG_R1: without force or with one along x).
+enum { MODE_FP = 0, MODE_EQ = 1, MODE_LEARNED = 2, MODE_SMAG = 3, MODE_FP_R1 = 4, MODE_EQ_R1 = 5, MODE_LEARNED_R1 = 6,
+       MODE_SMAG_R1 = 7 };
 
 // Body force of a step kernel: none, any, or along x only (the unit-rate modes have a collision of
 // their own for the last, see collide.cuh).
@@ -33,8 +35,10 @@ enum { FORCE_NONE = 0, FORCE_ANY = 1, FORCE_X = 2 };
 // FP or MCM attractors with the full register-cap / pipelined / paired variant set.
 __host__ __device__ constexpr bool plain_mode(int m) { return m == MODE_FP || m == MODE_EQ || m == MODE_FP_R1 || m == MODE_EQ_R1; }
 __host__ __device__ constexpr bool eq_mode(int m) { return m == MODE_EQ || m == MODE_EQ_R1; }
-__host__ __device__ constexpr bool r1_mode(int m) { return m == MODE_FP_R1 || m == MODE_EQ_R1 || m == MODE_LEARNED_R1; }
+__host__ __device__ constexpr bool r1_mode(int m) { return m == MODE_FP_R1 || m == MODE_EQ_R1 || m == MODE_LEARNED_R1 || m == MODE_SMAG_R1; }
 __host__ __device__ constexpr bool learned_mode(int m) { return m == MODE_LEARNED || m == MODE_LEARNED_R1; }
+
+__host__ __device__ constexpr bool smag_mode(int m) { return m == MODE_SMAG || m == MODE_SMAG_R1; }
 
 // Boundary kinds of the step kernel: periodic box; half-way bounce-back walls
 // at y = -1/2 and ny - 1/2 (x, z periodic); the same with the wall at
@@ -118,7 +122,7 @@ struct StepArgs {
     Rates<R> rates;
     int* flag;            // set to 1 by any cell with rho <= 0 or non-finite
     const float* closure; // packed MLP weights (learned mode), else null
-    const R* smag;        // (C_s Delta D(y))^2 per row y (Smagorinsky mode), else null
+    const void* smag;     // (C_s Delta D(y))^2 per row y in the arithmetic type (Smagorinsky modes), else null
 };
 
 // Storage traits: load as compute type R, store from R with round-to-nearest.

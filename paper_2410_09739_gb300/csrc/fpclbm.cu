@@ -176,7 +176,7 @@ StepArgs<R> make_args(const fpclbm* h)
     a.rates = make_rates<R>(h->omega);
     a.flag = h->d_flag;
     a.closure = h->d_closure;
-    a.smag = h->diffusion == FPCLBM_DIFF_FP_SMAGORINSKY ? static_cast<const R*>(h->d_smag) : nullptr;
+    a.smag = h->diffusion == FPCLBM_DIFF_FP_SMAGORINSKY ? h->d_smag : nullptr;
     return a;
 }
 
@@ -225,14 +225,15 @@ int force_kind(const fpclbm* h)
 // Collision mode of the step kernel.  A box or ensemble in the FP or MCM mode whose rates of
 // orders 3-6 (Step 3 indices 10..26) are all exactly 1 takes the unit-rate variant, which sets
 // those moments to their attractors plus half their sources (and, without force, never forms
-// their pre-collision values).
+// their pre-collision values); the Smagorinsky mode too, unless its force leaves the x axis.
 int mode_of(const fpclbm* h)
 {
-    if (h->diffusion == FPCLBM_DIFF_FP_SMAGORINSKY) return MODE_SMAG;
-    const int m = h->diffusion == FPCLBM_DIFF_FP_LEARNED ? MODE_LEARNED
+    const bool smag = h->diffusion == FPCLBM_DIFF_FP_SMAGORINSKY;
+    const int m = smag ? MODE_SMAG : h->diffusion == FPCLBM_DIFF_FP_LEARNED ? MODE_LEARNED
                   : h->diffusion == FPCLBM_DIFF_EQUILIBRIUM ? MODE_EQ : MODE_FP;
     for (int j = 10; j < 27; ++j)
         if (h->omega[j] != 1.0) return m;
+    if (smag) return force_kind(h) == FORCE_ANY ? MODE_SMAG : MODE_SMAG_R1;
     return m == MODE_EQ ? MODE_EQ_R1 : m == MODE_LEARNED ? MODE_LEARNED_R1 : MODE_FP_R1;
 }
 
@@ -438,6 +439,7 @@ int autotune(fpclbm* h)
                          (kb == BC_PERIODIC || kb == BC_WALLS_Y);
     // paired variant (two cells per thread, packed fp32): fp32 arithmetic, every boundary kind
     const bool pair_ok = fp32_math;
+    const bool pair_smag = h->precision != FPCLBM_FP64 && md == MODE_SMAG_R1;
     if (h->ensemble) {
         for (int minb : {2, 3})
             for (int block : {128, 256}) {
@@ -466,6 +468,7 @@ int autotune(fpclbm* h)
         for (int minb : {2, 1})
             for (int block : {128, 256}) cands.push_back({block, minb, 0, 0});
     } else {
+        if (pair_smag) cands.push_back({128, 2, 0, 2});
         for (int block : {128, 256}) cands.push_back({block, 1, 0, 0});
         if (pipe_ok) cands.push_back({128, 1, 0, 1});
     }
@@ -491,11 +494,12 @@ int autotune(fpclbm* h)
         if (forced.pipe == 3 && !stage_ok(h)) forced.pipe = pair_ok ? 2 : 0;
         const bool pair_learned = learned_mode(mode_of(h)) && h->precision != FPCLBM_FP64 &&
                                   (kb == BC_PERIODIC || kb == BC_WALLS_Y);
-        if ((forced.pipe == 1 && !pipe_ok) || (forced.pipe == 2 && !pair_ok && !pair_learned)) forced.pipe = 0;
+        if ((forced.pipe == 1 && !pipe_ok) || (forced.pipe == 2 && !pair_ok && !pair_learned && !pair_smag))
+            forced.pipe = 0;
         if (forced.pipe == 2 || forced.pipe == 3) forced.minb = 2;
         if (forced.pipe == 3) forced.block = stage_threads(h);
         if (forced.pipe != 3) forced.grid = 0;
-        if (!fp32_math && !learned_mode(mode_of(h))) forced.minb = 1;  // learned: 1 or 2 (else 1)
+        if (!fp32_math && !learned_mode(mode_of(h)) && forced.pipe != 2) forced.minb = 1;  // learned: 1 or 2 (else 1)
         h->block = forced.block;
         h->minb = forced.minb;
         h->grid = forced.grid;
@@ -807,9 +811,9 @@ int fpclbm_step(fpclbm_t h, long long n)
         const int kb = kernel_bc(h), md = mode_of(h);
         if (learned_mode(md) && !(kb == BC_PERIODIC || kb == BC_WALLS_Y))
             return fail(h, FPCLBM_ERR_ARG, "learned mode needs a periodic box or a channel with resting walls");
-        if (md == MODE_SMAG && !bc_fixed(kb))
+        if (smag_mode(md) && !bc_fixed(kb))
             return fail(h, FPCLBM_ERR_ARG, "Smagorinsky mode needs resting walls (no closed box, no moving wall)");
-        if (md == MODE_SMAG && h->smag_dirty) {
+        if (smag_mode(md) && h->smag_dirty) {
             int rc = upload_smag(h);
             if (rc) return rc;
         }
@@ -871,7 +875,7 @@ int fpclbm_get_launch(fpclbm_t h, int out[4])
     out[0] = h->block;
     out[1] = h->pipe == 3 ? h->grid : h->minb;  // variant 3: its shared-memory stages
     out[2] = h->pipe;
-    out[3] = mode_of(h);
+    out[3] = smag_mode(mode_of(h)) ? (int)MODE_SMAG : mode_of(h);  // one code for both Smagorinsky families
     return FPCLBM_OK;
 }
 

@@ -38,6 +38,7 @@ __device__ __forceinline__ bool operator<(f2 a, f2 b) { return a.v.x < b.v.x && 
 __device__ __forceinline__ f2 fminR(f2 a, f2 b) { return f2(fminf(a.v.x, b.v.x), fminf(a.v.y, b.v.y)); }
 __device__ __forceinline__ f2 fmaxR(f2 a, f2 b) { return f2(fmaxf(a.v.x, b.v.x), fmaxf(a.v.y, b.v.y)); }
 __device__ __forceinline__ f2 recipR(f2 a) { return f2(__frcp_rn(a.v.x), __frcp_rn(a.v.y)); }
+__device__ __forceinline__ f2 sqrtR(f2 a) { return f2(sqrtf(a.v.x), sqrtf(a.v.y)); }
 __device__ __forceinline__ f2 fmaR(f2 a, f2 b, f2 c) { return f2(__ffma2_rn(a.v, b.v, c.v)); }
 
 }  // namespace fpc
