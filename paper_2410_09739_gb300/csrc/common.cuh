@@ -157,6 +157,14 @@ struct Store<__nv_bfloat16> {
     __device__ __forceinline__ static __nv_bfloat16 fromd(double v) { return __double2bfloat16(v); }
 };
 
+// Chained steps (launch_chained in internal.h): a step kernel waits for its predecessor to have
+// finished, and its writes to be visible, before it touches the populations or the flag.  It never
+// signals the next one early (griddepcontrol.launch_dependents): the end of its blocks does, so only
+// the launch itself overlaps.  An early signal places the next grid's blocks while this one's still
+// run, unevenly over the SMs: an fp64 box of 32^3 cells, bound by the fp64 pipes of its fullest SM,
+// took 38 us a step instead of 27.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
 // 1D rest weights at e = -1, 0, +1 and rest central moments (1, 0, cs^2) per axis.
 __host__ __device__ constexpr double w1(int i) { return i == 1 ? 2.0 / 3.0 : 1.0 / 6.0; }
 __host__ __device__ constexpr double r1(int k) { return k == 0 ? 1.0 : (k == 1 ? 0.0 : 1.0 / 3.0); }

@@ -166,6 +166,7 @@ __global__ void __launch_bounds__(256) k_step2d(const Args2<R> a)
             yin[2] = y > 0;
         }
     }
+    chain_wait();
     R g[9];
 #pragma unroll
     for (int s = 0; s < 9; ++s) {
@@ -355,7 +356,7 @@ template <typename S, typename R, bool BOX>
 cudaError_t step2d_go(int odd, int force, int mode, const Args2<R>& a, cudaStream_t st)
 {
     const unsigned grid = (a.ncells + 255) / 256;
-#define FPC2_K(O, FO, M) k_step2d<S, R, O, FO, M, BOX><<<grid, 256, 0, st>>>(a)
+#define FPC2_K(O, FO, M) return launch_chained(k_step2d<S, R, O, FO, M, BOX>, grid, 256, 0, st, a)
     if (odd) {
         if (force) { if (mode == MODE_EQ) FPC2_K(true, true, MODE_EQ); else FPC2_K(true, true, MODE_FP); }
         else { if (mode == MODE_EQ) FPC2_K(true, false, MODE_EQ); else FPC2_K(true, false, MODE_FP); }
@@ -364,7 +365,6 @@ cudaError_t step2d_go(int odd, int force, int mode, const Args2<R>& a, cudaStrea
         else { if (mode == MODE_EQ) FPC2_K(false, false, MODE_EQ); else FPC2_K(false, false, MODE_FP); }
     }
 #undef FPC2_K
-    return cudaGetLastError();
 }
 
 constexpr int kGraph2 = 32;

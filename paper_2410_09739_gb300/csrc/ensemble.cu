@@ -42,6 +42,7 @@ template <bool ODD, int FORCE, int MODE, int MINB>
 __global__ void __launch_bounds__(256, MINB) k_ens_step(const EnsArgs a)
 {
     float* __restrict__ base = static_cast<float*>(a.buf);
+    chain_wait();
     for (unsigned t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
         const unsigned b = __ldg(a.tile_box + t);
         const EnsBox& B = a.boxes[b];
@@ -78,6 +79,7 @@ __global__ void __launch_bounds__(128, MINB) k_ens_pair(const EnsArgs a)
 {
     float* __restrict__ base = static_cast<float*>(a.buf);
     const unsigned half = a.tile_cells / 2;
+    chain_wait();
     for (unsigned t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
         const unsigned b = __ldg(a.tile_box + t);
         const EnsBox& B = a.boxes[b];
@@ -144,19 +146,13 @@ static cudaError_t go(const EnsArgs& a, int block, int minb, int grid, int varia
             // the persistent grid, sized by the tuner for the capped kernel, is scaled to match
             const int o = minb == 3 ? occ_even_pair<FORCE, MODE, 3>() : occ_even_pair<FORCE, MODE, 4>();
             const long long g5 = (long long)grid * occ_even_pair<FORCE, MODE, 5>() / o;
-            k_ens_pair<false, FORCE, MODE, 5><<<(unsigned)(g5 > 0 ? g5 : 1), block, 0, st>>>(a);
-            return cudaGetLastError();
+            return launch_chained(k_ens_pair<false, FORCE, MODE, 5>, (unsigned)(g5 > 0 ? g5 : 1), (unsigned)block, 0, st, a);
         }
-        if (minb == 3)
-            k_ens_pair<ODD, FORCE, MODE, 3><<<grid, block, 0, st>>>(a);
-        else
-            k_ens_pair<ODD, FORCE, MODE, 4><<<grid, block, 0, st>>>(a);
-    } else if (minb == 3) {
-        k_ens_step<ODD, FORCE, MODE, 3><<<grid, block, 0, st>>>(a);
-    } else {
-        k_ens_step<ODD, FORCE, MODE, 2><<<grid, block, 0, st>>>(a);
+        return launch_chained(minb == 3 ? k_ens_pair<ODD, FORCE, MODE, 3> : k_ens_pair<ODD, FORCE, MODE, 4>,
+                              (unsigned)grid, (unsigned)block, 0, st, a);
     }
-    return cudaGetLastError();
+    return launch_chained(minb == 3 ? k_ens_step<ODD, FORCE, MODE, 3> : k_ens_step<ODD, FORCE, MODE, 2>, (unsigned)grid,
+                          (unsigned)block, 0, st, a);
 }
 
 template <int MODE>

@@ -454,11 +454,17 @@ int autotune(fpclbm* h)
             cands.push_back({128, minb, (int)h->ntiles, 2});
         }
     } else if (fp32_math) {
+        // the first candidate runs boxes too small to tune: two cells per thread where the step is
+        // longer than its latency (fp32, us a step, one / two cells: 32^3 2.20 / 2.25, 48^3 4.56 /
+        // 3.59, 64^3 8.09 / 6.55, 96^3 29.8 / 23.8); rows of odd length pair cells c, c + N/2 and
+        // gain later (45x37x53 3.93 / 4.12, 63x65x67 8.6 / 7.9)
+        const unsigned long long pair_from = (h->boxes[0].nx & 1) ? 1ull << 18 : 1ull << 16;
+        if (h->total_cells >= pair_from) cands.push_back({128, 2, 0, 2});
         for (int minb : {2, 3, 4})
             for (int block : {128, 256}) cands.push_back({block, minb, 0, 0});
         if (pipe_ok)
             for (int minb : {2, 3, 4}) cands.push_back({128, minb, 0, 1});
-        if (pair_ok) cands.push_back({128, 2, 0, 2});  // 4 blocks of 128 threads, 128 registers
+        if (h->total_cells < pair_from) cands.push_back({128, 2, 0, 2});  // 4 blocks of 128 threads, 128 registers
         if (stage_ok(h))  // row-staged paired variant with 2 or 3 input stages
             for (int ns : {2, 3}) cands.push_back({stage_threads(h), 2, ns, 3});
     } else if (learned_mode(mode_of(h)) && h->precision != FPCLBM_FP64 && fixed_walls) {
@@ -469,6 +475,10 @@ int autotune(fpclbm* h)
             for (int block : {128, 256}) cands.push_back({block, minb, 0, 0});
     } else {
         if (pair_smag) cands.push_back({128, 2, 0, 2});
+        // fp64 first with blocks of one warp: the step is bound by the fp64 pipe of the SM with most
+        // cells, and small blocks share a small box out evenly (32^3, us a step with blocks of 128,
+        // 64, 32: 26.7, 26.6, 23.9; 16^3 14.2, 12.5, 12.6; equal from 45x37x53 on)
+        if (h->precision == FPCLBM_FP64) cands.push_back({32, 1, 0, 0});
         for (int block : {128, 256}) cands.push_back({block, 1, 0, 0});
         if (pipe_ok) cands.push_back({128, 1, 0, 1});
     }

@@ -366,6 +366,7 @@ __global__ void __launch_bounds__(32 * (NCW + 1), stage_min_blocks(NCW, FORCE, M
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         fence_proxy_async_smem();
     }
+    chain_wait();
     __syncthreads();
 
     // this CTA's tiles: t_i = blockIdx.x + i gridDim.x, i < nt
@@ -548,8 +549,8 @@ cudaError_t step_go_stage_ncw(const StepArgs<float>& a, int nsi, cudaStream_t st
     const unsigned ntiles = (unsigned)(a.ny / R) * (unsigned)a.nz;
     unsigned grid = (unsigned)(per_sm * sms);
     if (grid > ntiles) grid = ntiles;
-    kern<<<grid, threads, smem, st>>>(pair_args(a), make_fastdiv((unsigned)(a.ny / R)), ntiles, R, nsi);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, (unsigned)threads, smem, st, pair_args(a), make_fastdiv((unsigned)(a.ny / R)), ntiles,
+                          R, nsi);
 }
 
 // Tiles of up to 256 cells (4 consumer warps) for rows of at most 256 cells, of 384 (6 consumer

@@ -29,6 +29,7 @@ __global__ void __launch_bounds__(256, MINB) k_step(const StepArgs<R> a)
     G.div_nx = a.div_nx;
     G.div_nxny = a.div_nxny;
     const Rates<R>& rt = a.rates;
+    chain_wait();
     update_cell<S, R, ODD, BC, FORCE, MODE>(static_cast<S*>(a.buf), G, cell, rt, a.Fx, a.Fy, a.Fz,
                                             own_shear<FORCE, MODE>(rt), a.closure, a.flag, active,
                                             a.lid6x, a.lid6z, a.smag);
@@ -60,6 +61,7 @@ __device__ __forceinline__ void cp_async_wait()
 template <typename S, typename R, bool ODD, int BC, int FORCE, int MODE, int MINB>
 __global__ void __launch_bounds__(128, MINB) k_step_pipe(const StepArgs<R> a, unsigned ntiles)
 {
+    chain_wait();
     static_assert(sizeof(S) == 4 || sizeof(S) == 8, "cp.async moves 4, 8 or 16 bytes");
     static_assert(BC == BC_PERIODIC || BC == BC_WALLS_Y, "periodic or channel boxes only");
     static_assert(plain_mode(MODE), "FP and MCM modes only");
@@ -134,8 +136,7 @@ cudaError_t step_go_pipe(const StepArgs<R>& a, cudaStream_t st)
     const unsigned ntiles = (a.ncells + T - 1) / T;
     unsigned grid = (unsigned)(per_sm * sms);
     if (grid > ntiles) grid = ntiles;
-    kern<<<grid, T, smem, st>>>(a, ntiles);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, T, smem, st, a, ntiles);
 }
 
 // ---------------------------------------------------------------------------
@@ -166,6 +167,7 @@ __global__ void __launch_bounds__(128, MINB) k_step_pair(const StepArgs<f2> a, u
     G.div_nx = a.div_nx;
     G.div_nxny = a.div_nxny;
     const Rates<f2>& rt = a.rates;
+    chain_wait();
     if constexpr (ODD && ADJ)  // neighbouring cells 2 c1, 2 c1 + 1 with a shared neighbour table
         update_pair_odd_adj<S, BC, FORCE, MODE>(static_cast<S*>(a.buf), G, c1, rt, a.Fx, a.Fy, a.Fz,
                                                 own_shear<FORCE, MODE>(rt), a.flag, a.lid6x, a.lid6z, a.closure,
@@ -223,10 +225,8 @@ cudaError_t step_go_pair(const StepArgs<float>& a, cudaStream_t st)
     // fp32 storage (its per-cell x-wall tests spill with 16-bit unpacking)
     constexpr bool ADJ_OK = ODD && (BC != BC_BOX_LID || sizeof(S) == 4);
     if (ADJ_OK && (a.nx & 1) == 0)
-        k_step_pair<S, ODD, BC, FORCE, MODE, BLOCKS, ADJ_OK><<<grid, 128, 0, st>>>(pair_args(a), half);
-    else
-        k_step_pair<S, ODD, BC, FORCE, MODE, BLOCKS, false><<<grid, 128, 0, st>>>(pair_args(a), half);
-    return cudaGetLastError();
+        return launch_chained(k_step_pair<S, ODD, BC, FORCE, MODE, BLOCKS, ADJ_OK>, grid, 128, 0, st, pair_args(a), half);
+    return launch_chained(k_step_pair<S, ODD, BC, FORCE, MODE, BLOCKS, false>, grid, 128, 0, st, pair_args(a), half);
 }
 
 template <typename S, typename R, bool ODD, int BC, int FORCE, int MODE, int MINB>
@@ -254,8 +254,7 @@ cudaError_t step_go(const StepArgs<R>& a, const StepLaunch& cfg, cudaStream_t st
     }
     const int block = cfg.block > 0 ? cfg.block : 256;
     const unsigned grid = (a.ncells + block - 1) / block;
-    k_step<S, R, ODD, BC, FORCE, MODE, MINB><<<grid, block, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_step<S, R, ODD, BC, FORCE, MODE, MINB>, grid, (unsigned)block, 0, st, a);
 }
 
 // Register-cap variants exist for fp32 arithmetic: 2, 3, 4 for the FP and EQ
