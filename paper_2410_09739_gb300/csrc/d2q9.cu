@@ -8,8 +8,8 @@
 // odd step: neighbour gather / scatter), periodic in x and y or a closed
 // square box (half-way bounce-back on all four sides, the wall y = ny - 1/2
 // moving along x: the 2D lid-driven cavity of Sec. 4, handled as in 3D, see
-// cell.cuh).  One thread per cell: 9 loads, the collision in registers, 9
-// stores.
+// cell.cuh).  9 loads, the collision in registers, 9 stores per cell; one cell
+// per thread, or two on the packed fp32 pipe (k_step2d_pair).
 //
 // Collision (Step 3 of the 2D appendix) in deviation form: the central
 // moments come from two 3-point passes (y lines, then x lines; see fwd3 in
@@ -27,6 +27,7 @@
 
 #include "rtalloc.h"
 #include "aux.cuh"
+#include "cell.cuh"
 #include "collide.cuh"
 #include "field_math.cuh"
 #include "fpclbm.h"
@@ -53,9 +54,8 @@ struct Args2 {
     int* flag;
 };
 
-// 1D rest weights and rest central moments per axis index i = e + 1.
+// 1D rest weights per axis index i = e + 1.
 __host__ __device__ constexpr double w1d(int i) { return i == 1 ? 2.0 / 3.0 : 1.0 / 6.0; }
-__host__ __device__ constexpr double r1d(int k) { return k == 0 ? 1.0 : (k == 1 ? 0.0 : 1.0 / 3.0); }
 
 template <typename R, bool FORCE, int MODE>
 __device__ __forceinline__ bool collide2(R (&g)[9], const Rates2<R>& rt, R Fx, R Fy)
@@ -72,7 +72,7 @@ __device__ __forceinline__ bool collide2(R (&g)[9], const Rates2<R>& rt, R Fx, R
     const R jx = S[2] - S[0];
     const R jy = (Dy[0] + Dy[1]) + Dy[2];
     const R rho = R(1) + drho;
-    const R inv_rho = R(1) / rho;
+    const R inv_rho = recipR(rho);
     const bool ok = (rho > R(0)) && (rho < R(1e30));
     const R ux = (FORCE ? fmaR(R(0.5), Fx, jx) : jx) * inv_rho;
     const R uy = (FORCE ? fmaR(R(0.5), Fy, jy) : jy) * inv_rho;
@@ -196,6 +196,93 @@ __global__ void __launch_bounds__(256) k_step2d(const Args2<R> a)
         else
             p = buf + (size_t)s * stride + (xs[2 - ix] + ys[2 - iy]);
         Store<S>::st(p, g[s]);
+    }
+}
+
+// Two neighbouring cells c = 2t, c + 1 per thread on the packed fp32 pipe (pair.cuh), as in 3D
+// (update_pair_even, update_pair_odd_adj): half the arithmetic instructions, and every access whose
+// two values are adjacent (all of the even step, the three slots with e_x = 0 of the odd one) is one
+// vector access.  The odd step needs even nx: a pair then shares its row.  What bounds it is HBM
+// (fp32 4096^2: 181 us a step against 199 with one cell per thread; bf16 128 against 161).
+template <typename S, bool ODD, bool FORCE, int MODE, bool BOX>
+__global__ void __launch_bounds__(128) k_step2d_pair(const Args2<f2> a)
+{
+    const unsigned c = 2u * (blockIdx.x * blockDim.x + threadIdx.x);
+    if (c >= a.ncells) return;
+    const bool two = c + 1 < a.ncells;
+    S* __restrict__ buf = static_cast<S*>(a.buf);
+    const unsigned stride = a.stride, nx = a.nx, ny = a.ny;
+    unsigned x = 0, y = 0;
+    if (ODD || BOX) {
+        y = fdiv(c, a.div_nx);
+        x = c - y * nx;
+    }
+    // odd step: columns x - e_x of the two cells and row offsets y - e_y, e = -1, 0, +1
+    unsigned xa[3], xb[3], ys[3];
+    bool ina[3] = {true, true, true}, inb[3] = {true, true, true}, iny[3] = {true, true, true};
+    if (ODD) {
+        xa[0] = x + 1;
+        xa[1] = x;
+        xa[2] = x == 0 ? nx - 1 : x - 1;
+        xb[0] = x + 2 == nx ? 0u : x + 2;
+        xb[1] = x + 1;
+        xb[2] = x;
+        ys[0] = ((y + 1 == ny) ? 0u : y + 1) * nx;
+        ys[1] = y * nx;
+        ys[2] = ((y == 0) ? ny - 1 : y - 1) * nx;
+        if (BOX) {
+            ina[2] = x > 0;
+            inb[0] = x + 2 < nx;
+            iny[0] = y + 1 < ny;
+            iny[2] = y > 0;
+        }
+    }
+    chain_wait();
+    f2 g[9];
+#pragma unroll
+    for (int s = 0; s < 9; ++s) {
+        const int ix = s % 3, iy = s / 3;
+        const S *own = buf + (size_t)s * stride + c, *far = buf + (size_t)(8 - s) * stride;
+        if (!ODD) {
+            if (two) {
+                g[s] = Store2<S>::ld(own);
+            } else {
+                const float v = Store<S>::ld(own);
+                g[s] = f2(v, v);
+            }
+        } else if (ix == 1) {
+            g[s] = Store2<S>::ld(iny[iy] ? far + (x + ys[iy]) : own);
+        } else {
+            g[s].v.x = Store<S>::ld(ina[ix] && iny[iy] ? far + (xa[ix] + ys[iy]) : own);
+            g[s].v.y = Store<S>::ld(inb[ix] && iny[iy] ? far + (xb[ix] + ys[iy]) : own + 1);
+        }
+    }
+    const bool ok = collide2<f2, FORCE, MODE>(g, a.rt, a.Fx, a.Fy);
+    if (!ok) atomicOr(a.flag, 1);
+    if (BOX) {  // moving wall (k_step2d), the other lane's correction masked to zero
+        const bool ta = y + 1 == ny, tb = (x + 1 == nx ? y + 1 : y) + 1 == ny;
+        if (ta || tb) {
+            f2 rho = f2(1.0);
+#pragma unroll
+            for (int s = 0; s < 9; ++s) rho += g[s];
+            const f2 lid = a.lid6 * f2(ta ? 1.f : 0.f, tb ? 1.f : 0.f);
+            g[6] -= f2(w1d(0) * w1d(2)) * rho * (-lid);
+            g[8] -= f2(w1d(2) * w1d(2)) * rho * lid;
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < 9; ++s) {
+        const int ix = s % 3, iy = s / 3;
+        S *own = buf + (size_t)(8 - s) * stride + c, *far = buf + (size_t)s * stride;
+        if (!ODD) {
+            if (two) Store2<S>::st(own, g[s]);
+            else Store<S>::st(own, g[s].v.x);
+        } else if (ix == 1) {
+            Store2<S>::st(iny[2 - iy] ? far + (x + ys[2 - iy]) : own, g[s]);
+        } else {
+            Store<S>::st(ina[2 - ix] && iny[2 - iy] ? far + (xa[2 - ix] + ys[2 - iy]) : own, g[s].v.x);
+            Store<S>::st(inb[2 - ix] && iny[2 - iy] ? far + (xb[2 - ix] + ys[2 - iy]) : own + 1, g[s].v.y);
+        }
     }
 }
 
@@ -352,11 +439,46 @@ __global__ void k_set_pops2d(void* bufv, unsigned stride, unsigned n, const doub
     }
 }
 
+inline Args2<f2> pair_args(const Args2<float>& a)
+{
+    Args2<f2> p;
+    p.buf = a.buf;
+    p.stride = a.stride;
+    p.ncells = a.ncells;
+    p.nx = a.nx;
+    p.ny = a.ny;
+    p.div_nx = a.div_nx;
+    p.Fx = f2(a.Fx, a.Fx);
+    p.Fy = f2(a.Fy, a.Fy);
+    p.lid6 = f2(a.lid6, a.lid6);
+    for (int j = 0; j < 9; ++j) {
+        p.rt.om[j] = f2(a.rt.om[j], a.rt.om[j]);
+        p.rt.keep[j] = f2(a.rt.keep[j], a.rt.keep[j]);
+        p.rt.src[j] = f2(a.rt.src[j], a.rt.src[j]);
+    }
+    p.flag = a.flag;
+    return p;
+}
+
+// Boxes below this many cells run one cell per thread: their step is latency, not throughput
+// (256^2 fp32 2.0 us a step with one cell per thread, 64^2 1.7).
+constexpr unsigned kPair2Cells = 1u << 16;
+
+template <typename S, typename R, bool BOX, bool ODD, bool FORCE, int MODE>
+cudaError_t step2d_one(const Args2<R>& a, cudaStream_t st)
+{
+    if constexpr (sizeof(R) == 4) {  // fp32 arithmetic
+        if (a.ncells >= kPair2Cells && !(ODD && (a.nx & 1)))
+            return launch_chained(k_step2d_pair<S, ODD, FORCE, MODE, BOX>, ((a.ncells + 1) / 2 + 127) / 128, 128, 0, st,
+                                  pair_args(a));
+    }
+    return launch_chained(k_step2d<S, R, ODD, FORCE, MODE, BOX>, (a.ncells + 255) / 256, 256, 0, st, a);
+}
+
 template <typename S, typename R, bool BOX>
 cudaError_t step2d_go(int odd, int force, int mode, const Args2<R>& a, cudaStream_t st)
 {
-    const unsigned grid = (a.ncells + 255) / 256;
-#define FPC2_K(O, FO, M) return launch_chained(k_step2d<S, R, O, FO, M, BOX>, grid, 256, 0, st, a)
+#define FPC2_K(O, FO, M) return step2d_one<S, R, BOX, O, FO, M>(a, st)
     if (odd) {
         if (force) { if (mode == MODE_EQ) FPC2_K(true, true, MODE_EQ); else FPC2_K(true, true, MODE_FP); }
         else { if (mode == MODE_EQ) FPC2_K(true, false, MODE_EQ); else FPC2_K(true, false, MODE_FP); }
