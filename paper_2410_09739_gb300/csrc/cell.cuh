@@ -366,8 +366,8 @@ __device__ __forceinline__ void update_pair_odd_adj(S* __restrict__ buf, const C
             }
         }
     }
-    const bool ok = collide_cell<f2, FORCE, MODE>(g, rt, Fx, Fy, Fz, sh, closure,
-                                                  smag_pair<MODE>(G, c, c + 1, smag));
+    const bool ok = collide_cell<f2, FORCE, MODE, !r1_mode(MODE)>(g, rt, Fx, Fy, Fz, sh, closure,
+                                                                  smag_pair<MODE>(G, c, c + 1, smag));
     if (!active) return;
     if (!ok) atomicOr(flag, 1);
     asm volatile("" : "+r"(c));  // rebuild the store addresses (see update_cell)

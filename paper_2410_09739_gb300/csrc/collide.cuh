@@ -492,8 +492,9 @@ __device__ __forceinline__ bool collide_unit(R (&g)[27], const Rates<R>& rt, R F
     return ok;
 }
 
-// Any rates, any force: the central-moment transform of all 27 moments.
-template <typename R, int FORCE, int MODE>
+// Any rates, any force: the central-moment transform of all 27 moments.  NEWTON: the short reciprocal
+// (pair.cuh).
+template <typename R, int FORCE, int MODE, bool NEWTON>
 __device__ __forceinline__ bool collide_general(R (&g)[27], const Rates<R>& rt, R Fx, R Fy, R Fz, const Shear<R>& sh,
                                                 const float* closure, R c2)
 {
@@ -513,7 +514,9 @@ __device__ __forceinline__ bool collide_general(R (&g)[27], const Rates<R>& rt, 
     const R jy = ((S[6] - S[0]) + (S[7] - S[1])) + (S[8] - S[2]);
     const R jz = ((Dz[0] + Dz[1] + Dz[2]) + (Dz[3] + Dz[4] + Dz[5])) + (Dz[6] + Dz[7] + Dz[8]);
     const R rho = R(1) + drho;
-    const R inv_rho = recipR(rho);
+    R inv_rho;
+    if constexpr (NEWTON) inv_rho = recip_newton(rho);
+    else inv_rho = recipR(rho);
     const bool ok = (rho > R(0)) && (rho < R(1e30));
     R ux, uy, uz;
     if (FORCE) {
@@ -798,12 +801,12 @@ __device__ __forceinline__ bool collide_general(R (&g)[27], const Rates<R>& rt, 
 // sh: 1 minus the five shear rates (110, 101, 011, 2d1, 2d2; own_shear, or
 // an ensemble box's); closure: MLP weights (learned mode only); c2 = (C_s Delta D)^2 of the cell (Smagorinsky modes
 // only).  Returns false when rho <= 0 or not finite.
-template <typename R, int FORCE, int MODE>
+template <typename R, int FORCE, int MODE, bool NEWTON = false>
 __device__ __forceinline__ bool collide_cell(R (&g)[27], const Rates<R>& rt, R Fx, R Fy, R Fz, const Shear<R>& sh,
                                              const float* closure, R c2 = R(0))
 {
     if constexpr (unit_collision(FORCE, MODE)) return collide_unit<R, FORCE == FORCE_X, MODE>(g, rt, Fx, sh, closure, c2);
-    else return collide_general<R, FORCE, MODE>(g, rt, Fx, Fy, Fz, sh, closure, c2);
+    else return collide_general<R, FORCE, MODE, NEWTON>(g, rt, Fx, Fy, Fz, sh, closure, c2);
 }
 
 #undef FPC_PASS_B
