@@ -319,6 +319,39 @@ __device__ __forceinline__ void update_pair_even(S* __restrict__ buf, const Cell
     }
 }
 
+// Whether neither cell of the pair c, c + 1 (one row) has a link out of the box.
+__device__ __forceinline__ bool pair_inside(const CellGeom& G, unsigned c)
+{
+    const unsigned nxny = (unsigned)(G.nx * G.ny), z = fdiv(c, G.div_nxny), r = c - z * nxny;
+    const unsigned y = fdiv(r, G.div_nx), x = r - y * (unsigned)G.nx;
+    return x - 1u < (unsigned)G.nx - 3u && y - 1u < (unsigned)G.ny - 2u && z - 1u < (unsigned)G.nz - 2u &&
+           G.nx > 3 && G.ny > 2 && G.nz > 2;
+}
+
+// The odd step's reads (or, STORE, writes) of a pair with no link out of the box: the neighbour in
+// every slot row lies at a distance that is the same for all cells.
+template <typename S, bool STORE>
+__device__ __forceinline__ void move_inner(S* __restrict__ buf, const CellGeom& G, unsigned c, f2 (&g)[27])
+{
+    const int nx = G.nx, nxny = G.nx * G.ny;
+#pragma unroll
+    for (int s = 0; s < 27; ++s) {
+        const int ex = s % 3 - 1, d = ex + ((s / 3) % 3 - 1) * nx + (s / 9 - 1) * nxny;
+        S* p = buf + (STORE ? (long long)s * G.stride + d : (long long)(26 - s) * G.stride - d) + c;
+        if constexpr (STORE) {
+            if (ex == 0) {
+                Store2<S>::st(p, g[s]);
+            } else {
+                Store<S>::st(p, g[s].v.x);
+                Store<S>::st(p + 1, g[s].v.y);
+            }
+        } else {
+            if (ex == 0) g[s] = Store2<S>::ld(p);
+            else g[s] = f2(Store<S>::ld(p), Store<S>::ld(p + 1));
+        }
+    }
+}
+
 // Odd step of the paired kernel for boxes with nx even: neighbouring cells
 // c = 2t (x even) and c + 1 share y and z, hence the neighbour table.  For the
 // nine slots with e_x = 0 their two values (neighbour reads, bounce-back
@@ -340,7 +373,11 @@ __device__ __forceinline__ void update_pair_odd_adj(S* __restrict__ buf, const C
     const unsigned stride = G.stride;
     unsigned c = 2 * t;
     f2 g[27];
-    {
+    bool inner = false;  // closed box: no lane of the warp has a pair next to a wall
+    if constexpr (BC == BC_BOX_LID) inner = __all_sync(__activemask(), pair_inside(G, c));
+    if (inner) {
+        move_inner<S, false>(buf, G, c, g);
+    } else {
         const Nbr n = make_nbr<BC>(G, c);
         const int x = (int)n.xs[1];
         const int wp = x + 2 == G.nx ? -G.nx : 0;  // second cell's column x + 2 wraps
@@ -371,6 +408,10 @@ __device__ __forceinline__ void update_pair_odd_adj(S* __restrict__ buf, const C
     if (!active) return;
     if (!ok) atomicOr(flag, 1);
     asm volatile("" : "+r"(c));  // rebuild the store addresses (see update_cell)
+    if (inner) {
+        move_inner<S, true>(buf, G, c, g);
+        return;
+    }
     lid_correct_pair<BC>(g, G, c, c + 1, lid6x, lid6z);
     const Nbr n = make_nbr<BC>(G, c);
     const int x = (int)n.xs[1];
