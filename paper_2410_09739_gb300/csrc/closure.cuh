@@ -28,7 +28,7 @@ enum { CL_W1 = 0, CL_B1 = 576, CL_W2 = 640, CL_B2 = 4736, CL_W3 = 4800, CL_B3 = 
 //                 holds b1 (the A operand's input 9 is the constant 1)
 //   [512, 2560)   layer-2 B fragments: ((nt * 4 + kt) * 32 + lane) * 2 + {0, 1}
 //   [2560, 2624)  b1 (fp32), [2624, 2688) b2, [2688, 2752) W3, [2752] b3
-//   [2756, 3012)  layer-2 bias fragments: nt * 32 + lane, the first word of the B fragment of a
+//   [2756, 3012)  layer-2 bias fragments (not read by this kernel): nt * 32 + lane, the first word of the B fragment of a
 //                 K tile whose only non-zero row holds b2 (the second word is zero)
 // The weights, biases included, are bf16 values, so b1 and b2 enter the products exactly.
 enum { CP_F1 = 0, CP_F2 = 512, CP_B1 = 2560, CP_B2 = 2624, CP_W3 = 2688, CP_B3 = 2752, CP_F2B = 2756,
@@ -76,9 +76,10 @@ __device__ __forceinline__ uint2 ldg_pair(const uint32_t* p) { return __ldg(rein
 __device__ __forceinline__ float2 ldg_pair(const float* p) { return __ldg(reinterpret_cast<const float2*>(p)); }
 
 // delta omega of this lane's cell from its 9 inputs (warp-collective).  The warp's 32 cells form
-// two 16-row tiles; every weight fragment is loaded once and used by both tiles.  The biases enter
-// the products as weights of a constant input 1: b1 in the spare K column 9 of layer 1, b2 in a
-// fifth K tile of layer 2 whose A fragment is the constant 1 in column 64.
+// two 16-row tiles; every weight fragment is loaded once and used by both tiles.  b1 enters layer 1's
+// product as the weight of a constant input 1 in the spare K column 9; b2 is the accumulator input of
+// layer 2's first product (a fifth K tile for it cost 16 of 96 products a warp) and the output layer
+// runs on packed pairs of columns: 192x96x96 bf16 channel 120 + 101 us a step pair before, 117 + 96 now.
 template <typename R>
 __device__ R closure_delta_omega(const uint32_t* __restrict__ P, const R in[9])
 {
@@ -124,37 +125,35 @@ __device__ R closure_delta_omega(const uint32_t* __restrict__ P, const R in[9])
             A2[mt][kt][h + 1] = pack_bf16x2(tanh_mufu(c[2]), tanh_mufu(c[3]));  // row g+8
         }
     }
-    // layer 2 (b2 first, through the constant-1 K tile) + tanh + output-layer partial sums over
-    // this lane's columns 2t, 2t+1 of each n-tile
-    const uint32_t one = t == 0 ? pack_bf16x2(1.f, 0.f) : 0u;  // A fragment: 1 in K column 64
-    const uint32_t aone[4] = {one, one, 0u, 0u};
-    float ylo[2] = {0.f, 0.f}, yhi[2] = {0.f, 0.f};
+    // layer 2 (b2 as the first product's accumulator input) + tanh + output-layer partial sums over
+    // this lane's columns 2t, 2t+1 of each n-tile, both columns of a row in one packed fma
+    f2 ylo[2] = {f2(0.f, 0.f), f2(0.f, 0.f)}, yhi[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
         const int n0 = 8 * nt + 2 * t;
-        const uint2 bias = make_uint2(__ldg(P + CP_F2B + nt * 32 + lane), 0u);
+        const float2 b2 = ldg_pair(Pf + CP_B2 + n0);
         float c[2][4];
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt) mma_bf16_16816(c[mt], aone, bias, 0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int kt = 0; kt < 4; ++kt) {
             const uint2 b = ldg_pair(P + CP_F2 + ((nt * 4 + kt) * 32 + lane) * 2);
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
-                mma_bf16_16816(c[mt], A2[mt][kt], b, c[mt][0], c[mt][1], c[mt][2], c[mt][3]);
+            for (int mt = 0; mt < 2; ++mt) {
+                if (kt == 0) mma_bf16_16816(c[mt], A2[mt][kt], b, b2.x, b2.y, b2.x, b2.y);
+                else mma_bf16_16816(c[mt], A2[mt][kt], b, c[mt][0], c[mt][1], c[mt][2], c[mt][3]);
+            }
         }
-        const float2 w = ldg_pair(Pf + CP_W3 + n0);
+        const f2 w = f2(ldg_pair(Pf + CP_W3 + n0));
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt) {
-            ylo[mt] = fmaf(w.x, tanh_mufu(c[mt][0]), fmaf(w.y, tanh_mufu(c[mt][1]), ylo[mt]));
-            yhi[mt] = fmaf(w.x, tanh_mufu(c[mt][2]), fmaf(w.y, tanh_mufu(c[mt][3]), yhi[mt]));
+            ylo[mt] = fmaR(w, f2(tanh_mufu(c[mt][0]), tanh_mufu(c[mt][1])), ylo[mt]);
+            yhi[mt] = fmaR(w, f2(tanh_mufu(c[mt][2]), tanh_mufu(c[mt][3])), yhi[mt]);
         }
     }
     // sum over the quad (the 4 lanes sharing rows g, g+8), then hand row r of tile mt to lane 16 mt + r
     float mine = 0.f;
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt) {
-        float lo = ylo[mt], hi = yhi[mt];
+        float lo = ylo[mt].v.x + ylo[mt].v.y, hi = yhi[mt].v.x + yhi[mt].v.y;
         lo += __shfl_xor_sync(0xffffffffu, lo, 1);
         lo += __shfl_xor_sync(0xffffffffu, lo, 2);
         hi += __shfl_xor_sync(0xffffffffu, hi, 1);
