@@ -4,6 +4,7 @@
 // where k_init_eq and k_moments state otherwise for fp32 and 16-bit storage.
 #include "aux.cuh"
 #include "field_math.cuh"
+#include "handle.h"
 #include "internal.h"
 
 namespace fpc {
@@ -107,12 +108,11 @@ __global__ void k_init_eq(BoxGeom b, const double* rho, const double* ux, const 
     }
 }
 
-// FP32 storage: cells c0 + 2i and c0 + 2i + 1 in the lanes of f2 values (c0 is even, so the two
-// entries of a slot are one 8-byte store).
-__global__ void __launch_bounds__(128) k_init_eq_pair(BoxGeom b, const double* rho, const double* ux,
-                                                      const double* uy, const double* uz, unsigned c0, unsigned n)
+// FP32 storage: cells c0 + i and c0 + i + 1 (i, c0 even) in the lanes of f2 values, so the two
+// entries of a slot are one 8-byte store.  The fields start at cell c0; n of its cells are in range.
+__device__ __forceinline__ void init_pair(const BoxGeom& b, const double* rho, const double* ux, const double* uy,
+                                          const double* uz, unsigned c0, unsigned i, unsigned n)
 {
-    const unsigned i = 2u * (blockIdx.x * blockDim.x + threadIdx.x);
     if (i >= n) return;
     const bool two = i + 1 < n;
     const unsigned j = two ? i + 1 : i, cell = c0 + i;
@@ -153,6 +153,44 @@ __global__ void __launch_bounds__(128) k_init_eq_pair(BoxGeom b, const double* r
         }
 }
 
+__global__ void __launch_bounds__(128) k_init_eq_pair(BoxGeom b, const double* rho, const double* ux,
+                                                      const double* uy, const double* uz, unsigned c0, unsigned n)
+{
+    init_pair(b, rho, ux, uy, uz, c0, 2u * (blockIdx.x * blockDim.x + threadIdx.x), n);
+}
+
+// Geometry of an ensemble's box.
+__device__ __forceinline__ BoxGeom ens_geom(const EnsArgs& a, const EnsBox& B)
+{
+    BoxGeom g;
+    g.buf = static_cast<float*>(a.buf) + __ldg(&B.off);
+    g.stride = __ldg(&B.stride);
+    g.ncells = __ldg(&B.ncells);
+    g.nx = __ldg(&B.nx);
+    g.ny = __ldg(&B.ny);
+    g.nz = __ldg(&B.nz);
+    g.walls = 0;
+    g.div_nx.d = __ldg(&B.div_nx.d);
+    g.div_nx.m = __ldg(&B.div_nx.m);
+    g.div_nx.s = __ldg(&B.div_nx.s);
+    g.div_nxny.d = __ldg(&B.div_nxny.d);
+    g.div_nxny.m = __ldg(&B.div_nxny.m);
+    g.div_nxny.s = __ldg(&B.div_nxny.s);
+    return g;
+}
+
+// All boxes of an ensemble: a block takes a tile of 256 cells.  (One launch per box left the chip
+// partly empty at the end of each: 0.83 ms in and 0.90 ms out against 0.58 and 0.70 now for 64 boxes of 32^3 to 96^3 cells.)
+__global__ void __launch_bounds__(128) k_init_eq_ens(const EnsArgs a, const double* rho, const double* ux,
+                                                     const double* uy, const double* uz)
+{
+    const EnsBox& B = a.boxes[__ldg(a.tile_box + blockIdx.x)];
+    const unsigned first = (blockIdx.x - __ldg(&B.tile0)) * a.tile_cells, cell0 = __ldg(&B.cell0);
+    const BoxGeom g = ens_geom(a, B);
+    for (unsigned i = first + 2u * threadIdx.x; i < first + a.tile_cells; i += 2u * blockDim.x)
+        init_pair(g, rho + cell0, ux + cell0, uy + cell0, uz + cell0, 0, i, g.ncells);
+}
+
 // Density and half-force velocity (Step 7) of every cell, in fp64.  For fp32
 // and 16-bit storage the 27 deviations are summed in fp32 with compensation
 // (sum2_add), which gives the fp64 sums in all but the last bits at fp32 cost,
@@ -161,11 +199,10 @@ __global__ void __launch_bounds__(128) k_init_eq_pair(BoxGeom b, const double* r
 // (field_math.cuh) bounds the kernel with every operation it is given, 0.75 ms for 256^3 cells before and 0.52 ms now (bf16: 0.75 and 0.51).
 // FP64 storage keeps the fp64 form.  has_force: any of the force is not zero.
 template <typename S>
-__global__ void k_moments(BoxGeom b, int parity, int has_force, double Fx, double Fy, double Fz, double* rho, double* ux,
-                          double* uy, double* uz, unsigned c0, unsigned n)
+__device__ __forceinline__ void moments_cell(const BoxGeom& b, int parity, int has_force, double Fx, double Fy,
+                                             double Fz, double* rho, double* ux, double* uy, double* uz, unsigned c0,
+                                             unsigned i)
 {
-    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
     if constexpr (!std::is_same<S, double>::value) {
         float g[27];
         load_cell<S>(b, parity, c0 + i, g);
@@ -206,6 +243,26 @@ __global__ void k_moments(BoxGeom b, int parity, int has_force, double Fx, doubl
     if (ux) ux[i] = (jx + 0.5 * Fx) / r;
     if (uy) uy[i] = (jy + 0.5 * Fy) / r;
     if (uz) uz[i] = (jz + 0.5 * Fz) / r;
+}
+
+template <typename S>
+__global__ void k_moments(BoxGeom b, int parity, int has_force, double Fx, double Fy, double Fz, double* rho,
+                          double* ux, double* uy, double* uz, unsigned c0, unsigned n)
+{
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) moments_cell<S>(b, parity, has_force, Fx, Fy, Fz, rho, ux, uy, uz, c0, i);
+}
+
+__global__ void __launch_bounds__(256) k_moments_ens(const EnsArgs a, int parity, int has_force, double Fx, double Fy,
+                                                     double Fz, double* rho, double* ux, double* uy, double* uz)
+{
+    const EnsBox& B = a.boxes[__ldg(a.tile_box + blockIdx.x)];
+    const unsigned first = (blockIdx.x - __ldg(&B.tile0)) * a.tile_cells, cell0 = __ldg(&B.cell0);
+    const BoxGeom g = ens_geom(a, B);
+    const unsigned end = min(first + a.tile_cells, g.ncells);
+    for (unsigned i = first + threadIdx.x; i < end; i += blockDim.x)
+        moments_cell<float>(g, parity, has_force, Fx, Fy, Fz, rho ? rho + cell0 : nullptr, ux ? ux + cell0 : nullptr,
+                            uy ? uy + cell0 : nullptr, uz ? uz + cell0 : nullptr, 0, i);
 }
 
 template <typename S>
@@ -351,6 +408,21 @@ cudaError_t launch_moments(int precision, const BoxGeom& b, int parity, double F
     const int force = Fx != 0.0 || Fy != 0.0 || Fz != 0.0;
     FPC_DISPATCH(precision, (k_moments<S><<<blocks_for(n, 256), 256, 0, st>>>(b, parity, force, Fx, Fy, Fz, rho, ux, uy,
                                                                               uz, c0, n)));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_init_eq_ens(const EnsArgs& a, const double* rho, const double* ux, const double* uy,
+                               const double* uz, cudaStream_t st)
+{
+    k_init_eq_ens<<<a.ntiles, 128, 0, st>>>(a, rho, ux, uy, uz);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_moments_ens(const EnsArgs& a, int parity, const double F[3], double* rho, double* ux, double* uy,
+                               double* uz, cudaStream_t st)
+{
+    const int force = F[0] != 0.0 || F[1] != 0.0 || F[2] != 0.0;
+    k_moments_ens<<<a.ntiles, 256, 0, st>>>(a, parity, force, F[0], F[1], F[2], rho, ux, uy, uz);
     return cudaGetLastError();
 }
 

@@ -308,6 +308,7 @@ extern "C" int fpclbm_create_ensemble(fpclbm_t* out, int n_boxes, const int* dim
                 E.keep4 = (float)(keep / 4);
                 E.keep6 = (float)(keep / 6);
                 E.tile0 = bx.tile0;
+                E.cell0 = bx.cell0;
                 for (unsigned t = 0; t < bx.ntiles; ++t) tb[bx.tile0 + t] = (unsigned)b;
             }
             e = cudaMemcpyAsync(h->d_ens_boxes, tab.data(), sizeof(EnsBox) * n_boxes, cudaMemcpyHostToDevice,

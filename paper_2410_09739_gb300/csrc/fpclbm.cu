@@ -691,7 +691,10 @@ int fpclbm_init_fields(fpclbm_t h, const double* rho, const double* ux, const do
             on_device = 1;
         }
     }
+    if (h->ensemble && on_device)  // all boxes at once
+        FPC_CK(h, launch_init_eq_ens(make_ens_args(h), rho, ux, uy, uz, h->stream), "init kernel");
     for (const Box& b : h->boxes) {
+        if (h->ensemble && on_device) break;
         const BoxGeom g = geom_of(h, b);
         if (on_device) {
             FPC_CK(h,
@@ -908,7 +911,11 @@ int fpclbm_moments(fpclbm_t h, double* rho, double* ux, double* uy, double* uz, 
             on_device = 1;
         }
     }
+    if (h->ensemble && on_device)  // all boxes at once
+        FPC_CK(h, launch_moments_ens(make_ens_args(h), parity, h->F, outs[0], outs[1], outs[2], outs[3], h->stream),
+               "moments kernel");
     for (const Box& b : h->boxes) {
+        if (h->ensemble && on_device) break;
         const BoxGeom g = geom_of(h, b);
         if (on_device) {
             double* o[4];

@@ -32,7 +32,7 @@ struct EnsBox {
     int nx, ny, nz;
     FastDiv div_nx, div_nxny;
     float keep, keep4, keep6;  // 1 - omega of the box's shear rate, and that over 4 and over 6
-    unsigned tile0;
+    unsigned tile0, cell0;     // first tile, first cell of the concatenated field arrays
 };
 
 struct EnsArgs {
@@ -53,6 +53,13 @@ struct EnsArgs {
 cudaError_t launch_ens_step(int odd, int force, int mode, const EnsArgs& a, int block, int minb, int grid,
                             int variant, cudaStream_t st);
 int ens_max_blocks_per_sm(int block, int minb, int mode, int variant);
+
+// launch_init_eq and launch_moments (internal.h) of all boxes of an ensemble (fp32 storage) in one
+// launch each; the field arrays are the concatenated ones of the C ABI.
+cudaError_t launch_init_eq_ens(const EnsArgs& a, const double* rho, const double* ux, const double* uy,
+                               const double* uz, cudaStream_t st);
+cudaError_t launch_moments_ens(const EnsArgs& a, int parity, const double F[3], double* rho, double* ux, double* uy,
+                               double* uz, cudaStream_t st);
 
 }  // namespace fpc
 

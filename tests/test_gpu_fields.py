@@ -104,3 +104,40 @@ def test_extreme_cells_take_the_fp64_form():
     scale = np.max(np.abs(f[:, ordinary]), axis=0)
     assert np.all(np.abs(got[:, ordinary] - f[:, ordinary]) <= 2.0 ** -24 * np.abs(f[:, ordinary]) + 2.0 ** -45 * scale)
     assert not np.any(np.isfinite(got[:, [3, 4, 7]]).all(axis=0))
+
+
+def test_ensemble_fields_on_the_device_equal_single_boxes():
+    """Fields in and out of an ensemble in one launch each, boxes of odd sizes (odd offsets in the
+    concatenated arrays, ragged tiles): the same populations and moments as single boxes."""
+    torch = pytest.importorskip("torch")
+    dims = [(7, 5, 3), (16, 9, 2), (1, 1, 1), (31, 3, 3), (40, 7, 5)]
+    taus = [0.6, 0.7, 0.8, 0.9, 1.0]
+    flds = [W.random_fields(*d, seed=20 + i) for i, d in enumerate(dims)]
+    flat = [torch.from_numpy(np.concatenate([f[q].ravel() for f in flds])).cuda() for q in range(4)]
+    for steps in (0, 3):
+        with F.Lattice.ensemble(dims, taus, "fp32") as ens:
+            ens.set_force(1e-4, 0.0, -1e-4)
+            F.fpclbm_init_fields(ens.h, *flat, on_device=1)
+            ens.step(steps)
+            out = [torch.full((ens.ncells,), np.nan, dtype=torch.float64, device="cuda") for _ in range(4)]
+            F.fpclbm_moments(ens.h, *out, on_device=1)
+            only = torch.full((ens.ncells,), np.nan, dtype=torch.float64, device="cuda")
+            from ctypes import c_void_p
+            assert F.load().fpclbm_moments(ens.h, None, None, c_void_p(only.data_ptr()), None, 1) == 0
+            f = ens.get_populations()
+        assert torch.equal(only, out[2])
+        at = 0
+        for d, tau, fl in zip(dims, taus, flds):
+            n = d[0] * d[1] * d[2]
+            with F.Lattice(*d, "fp32") as one:
+                one.set_params(tau)
+                one.set_force(1e-4, 0.0, -1e-4)
+                one.init_fields(*fl)
+                g = one.get_populations().reshape(27, -1)
+                if steps == 0:
+                    assert np.array_equal(f[:, at:at + n], g)
+                one.set_populations(f[:, at:at + n])
+                ref = one.moments()
+            for a, b in zip(out, ref):
+                assert np.max(np.abs(a[at:at + n].cpu().numpy() - b.ravel())) <= 1e-7
+            at += n
