@@ -218,10 +218,14 @@ cudaError_t step_go_pair(const StepArgs<float>& a, cudaStream_t st)
     // the even step without force or moving wall (vector accesses, no neighbour table, no source
     // terms) fits in 96 registers without spilling: one block more per SM.  With a force along x it
     // spills 28 bytes there and is faster all the same (384x192x192 bf16 channel: 326 -> 281 us;
-    // fp32, bound by HBM: unchanged).  The learned modes run
-    // four blocks (128 registers, about 90 bytes of spills: 2.5 % faster than three blocks at 168)
+    // fp32, bound by HBM: unchanged); 16-bit storage gains from the fifth block on the odd step too
+    // (148 bytes of spills; same channel 402 -> 384 us; not the fp32 LES, 177 -> 179).  The learned
+    // modes run four blocks (128 registers, about 90 bytes of spills: 2.5 % faster than three blocks
+    // at 168)
     constexpr bool LID = BC == BC_WALLS_Y_LID || BC == BC_BOX_LID;
-    constexpr int BLOCKS = learned_mode(MODE) ? 4 : (ODD || FORCE == FORCE_ANY || LID) ? 2 * MINB : 2 * MINB + 1;
+    constexpr bool WIDE_ODD = FORCE == FORCE_X && sizeof(S) == 2 && plain_mode(MODE);
+    constexpr bool NARROW = (ODD && !WIDE_ODD) || FORCE == FORCE_ANY || LID;
+    constexpr int BLOCKS = learned_mode(MODE) ? 4 : NARROW ? 2 * MINB : 2 * MINB + 1;
     const unsigned grid = (half + 127) / 128;
     // neighbouring cells on the odd step: nx even (rows hold whole pairs); the closed box only with
     // fp32 storage (its per-cell x-wall tests spill with 16-bit unpacking)
