@@ -520,7 +520,9 @@ int autotune(fpclbm* h)
         std::lock_guard<std::mutex> lk(g_tune_mu);
         load_tune_file();
         auto it = g_tune_cache.find(tune_key(h));
-        if (it != g_tune_cache.end()) {
+        // the key holds the cell count, not the row length: a row-staged choice of another box is no
+        // choice for one whose rows cannot be staged
+        if (it != g_tune_cache.end() && (it->second.pipe != 3 || stage_ok(h))) {
             h->block = it->second.block;
             h->minb = it->second.minb;
             h->grid = it->second.grid;

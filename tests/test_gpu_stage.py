@@ -139,3 +139,16 @@ def test_stage_full_size_bf16_tgv_256_matches_paired(monkeypatch):
             assert lat.launch()["variant"] == int(launch[-1])
             out.append(lat.populations_at(cells))
     assert np.array_equal(out[0], out[1])
+
+
+def test_tuned_choice_of_another_row_length():
+    """Two boxes of the same tuning key (precision, boundary, rates, 2^20 cells), the second with rows
+    that bulk copies cannot move (130 bf16 values are not a multiple of 16 bytes): the first one's
+    tuned choice may be the row-staged kernel, and the second must still step."""
+    for shape in ((128, 128, 64), (130, 126, 65)):
+        nx, ny, nz = shape
+        with F.Lattice(nx, ny, nz, "bf16") as lat:
+            lat.set_params(0.7)
+            lat.init_fields(*W.random_fields(nx, ny, nz, 1, u_amp=0.02))
+            lat.step(2)
+            assert nx % 8 == 0 or lat.launch()["variant"] != 3
