@@ -215,8 +215,8 @@ __global__ void k_cl_label(const double* __restrict__ acc, int cx, int cy, int c
 // tiles each, scalar transposes and 8-way bank conflicts took 17.2 us for it.
 //
 // Two kernels run the tiles:
-//   k_cl_epoch  batches of up to kMaxCluster tiles: one cluster of blocks runs all batches of an
-//               epoch, a tile per block.  The gradients go straight into the shared memory of the
+//   k_cl_epoch  batches of up to kMaxCluster tiles: one cluster of blocks runs up to kEpochBatches
+//               batches in a launch, a tile per block.  The gradients go straight into the shared memory of the
 //               block that owns the parameter, which sums them in block order, applies Adam to its
 //               fp32 master weights there and writes the new bf16 weight into every block's copy;
 //               two cluster barriers per batch, no launch and no global memory but the samples
@@ -555,17 +555,25 @@ __device__ __forceinline__ float adam(float w, float& m, float& v, float g, floa
     return w - lr * (mm * c1) / (sqrtf(vv * c2) + eps);
 }
 
-// An epoch on one cluster (gridDim.x = cluster size = tiles of a full batch, at most kMaxCluster).
+// Up to kEpochBatches consecutive batches of an epoch on one cluster (gridDim.x = cluster size = tiles
+// of a full batch, at most kMaxCluster).  Adam's bias corrections come as kernel arguments, as
+// k_cl_reduce_adam's do: they are exact host values, and no host buffer has to outlive the launch.
+// 256 of them keep the arguments under 4 KB, and a launch under a few milliseconds whatever the
+// number of batches (2.6 ms for 256 batches of 1,024 samples).
+constexpr int kEpochBatches = 256;
+
 struct EpochArgs {
-    NetArgs net;               // X, T, n, epoch order, standardisation, W (initial bf16 weights)
-    long long batch, batches;  // samples per batch, batches of the epoch
-    const float2* corr;        // Adam's bias corrections (c1, c2) of every batch
+    NetArgs net;              // X, T, n, epoch order, standardisation, W (bf16 weights before the first batch)
+    long long batch, first;   // samples per batch, first batch of this launch
+    int batches;              // batches of this launch, at most kEpochBatches
     float lr, b1, b2, eps;
-    float *w, *m, *v;          // fp32 master weights and moments, in place
-    __nv_bfloat16* wb;         // bf16 weights, out
-    double* loss;              // sum of squared errors of the epoch, added
-    FastDiv chunk;             // parameters owned by a block
+    float *w, *m, *v;         // fp32 master weights and moments, in place
+    __nv_bfloat16* wb;        // bf16 weights, out
+    double* loss;             // sum of squared errors of the epoch, continued
+    FastDiv chunk;            // parameters owned by a block
+    float2 corr[kEpochBatches];  // Adam's bias corrections (c1, c2) of every batch
 };
+static_assert(sizeof(EpochArgs) <= 4096, "kernel arguments");
 
 // Shared memory behind the tile's tables: received gradients [tiles][chunk], received losses, the
 // owned parameters' master weights and moments.
@@ -600,7 +608,7 @@ __device__ __forceinline__ void cluster_barrier()
     asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;\n" ::: "memory");
 }
 
-__global__ void __launch_bounds__(kTrainThreads) k_cl_epoch(const EpochArgs a)
+__global__ void __launch_bounds__(kTrainThreads) k_cl_epoch(const __grid_constant__ EpochArgs a)
 {
     extern __shared__ __align__(16) unsigned char cl_smem[];
     TrainSmem& S = *reinterpret_cast<TrainSmem*>(cl_smem);
@@ -617,17 +625,19 @@ __global__ void __launch_bounds__(kTrainThreads) k_cl_epoch(const EpochArgs a)
     }
     train_setup(S, a.net.W);
     const unsigned long long n = a.net.n;
-    auto fetch = [&](long long it) {
-        const unsigned long long first = (unsigned long long)(it * a.batch);
+    auto fetch = [&](int it) {
+        const unsigned long long first = (unsigned long long)((a.first + it) * a.batch);
         const unsigned long long end = min(first + (unsigned long long)a.batch, n);
         return load_sample(a.net, it < a.batches ? first + (unsigned long long)rank * kMB + tid : end, end);
     };
     Sample s;
     if (tid < kMB) s = fetch(0);
-    double loss = 0.0;
+    // one chain of additions over the batches of an epoch, whatever launches it takes
+    const bool sums_loss = rank == 0 && tid == kTrainThreads - 1;
+    double loss = sums_loss ? *a.loss : 0.0;
     cluster_barrier();  // every block's tables are in place before another one writes to them
-    for (long long it = 0; it < a.batches; ++it) {
-        const long long first = it * a.batch;
+    for (int it = 0; it < a.batches; ++it) {
+        const long long first = (a.first + it) * a.batch;
         const long long count = min((long long)n - first, a.batch);
         const unsigned tiles = (unsigned)((count + kMB - 1) / kMB);
         if (rank < tiles) {
@@ -660,7 +670,7 @@ __global__ void __launch_bounds__(kTrainThreads) k_cl_epoch(const EpochArgs a)
                 for (unsigned b = 0; b < nb; ++b) cluster_st(cluster_addr(at, b), __bfloat162float(wb));
             }
         }
-        if (rank == 0 && tid == kTrainThreads - 1) {
+        if (sums_loss) {
             double l = 0.0;
             for (unsigned b = 0; b < tiles; ++b) l += recv_loss[b];
             loss += l;
@@ -673,7 +683,7 @@ __global__ void __launch_bounds__(kTrainThreads) k_cl_epoch(const EpochArgs a)
         a.v[p0 + i] = mv[i];
         a.wb[p0 + i] = __float2bfloat16_rn(mw[i]);
     }
-    if (rank == 0 && tid == kTrainThreads - 1) *a.loss += loss;
+    if (sums_loss) *a.loss = loss;
 }
 
 // Second stage: sum of the block gradients in block order; the loss (fp64) is added to *loss.
@@ -1012,14 +1022,11 @@ extern "C" int fpclbm_closure_train(const float* X, const float* T, long long n,
     float *dw = nullptr, *dm = nullptr, *dv = nullptr, *dP = nullptr;
     __nv_bfloat16* dwb = nullptr;
     double *dL = nullptr, *dPL = nullptr;
-    float2* dC = nullptr;
     const long long batches = (n + batch - 1) / batch;
     EpochArgs ea;
     std::memset(&ea, 0, sizeof ea);
-    bool cluster = false;  // batches of few tiles: an epoch is one launch of one cluster
+    bool cluster = false;  // batches of few tiles: one cluster runs many of them in a launch
     e = epoch_launch(ea, max_blocks, st, true, &cluster);
-    std::vector<float2> corr(cluster ? (size_t)batches : 0);
-    if (e == cudaSuccess && cluster) e = rt_malloc(&dC, sizeof(float2) * (size_t)batches);
     if (e == cudaSuccess) e = rt_malloc(&dw, sizeof(float) * CL_N);
     if (e == cudaSuccess) e = rt_malloc(&dm, sizeof(float) * CL_N);
     if (e == cudaSuccess) e = rt_malloc(&dv, sizeof(float) * CL_N);
@@ -1035,7 +1042,6 @@ extern "C" int fpclbm_closure_train(const float* X, const float* T, long long n,
         rt_free(dPL);
         rt_free(dwb);
         rt_free(dL);
-        rt_free(dC);
     };
     if (e != cudaSuccess) {
         cleanup();
@@ -1066,8 +1072,6 @@ extern "C" int fpclbm_closure_train(const float* X, const float* T, long long n,
     };
     if (cluster) {
         ea.batch = std::min<long long>(batch, n);
-        ea.batches = batches;
-        ea.corr = dC;
         ea.lr = (float)lr;
         ea.b1 = b1;
         ea.b2 = b2;
@@ -1086,13 +1090,12 @@ extern "C" int fpclbm_closure_train(const float* X, const float* T, long long n,
         a.perm_a = pa;
         a.perm_c = splitmix(rs) % (uint64_t)n;
         e = cudaMemsetAsync(dL, 0, sizeof(double), st);
-        if (cluster && e == cudaSuccess) {
-            for (long long k = 0; k < batches; ++k) corr[(size_t)k] = correction(step + k + 1);
-            step += batches;
-            // pageable source: the copy has left the host buffer when the call returns
-            e = cudaMemcpyAsync(dC, corr.data(), sizeof(float2) * (size_t)batches, cudaMemcpyHostToDevice, st);
-            ea.net = a;
-            if (e == cudaSuccess) e = epoch_launch(ea, max_blocks, st, false, nullptr);
+        ea.net = a;
+        for (long long b = 0; cluster && b < batches && e == cudaSuccess; b += ea.batches) {
+            ea.first = b;
+            ea.batches = (int)std::min<long long>(batches - b, kEpochBatches);
+            for (int k = 0; k < ea.batches; ++k) ea.corr[k] = correction(++step);
+            e = epoch_launch(ea, max_blocks, st, false, nullptr);
         }
         for (long long first = 0; !cluster && first < n && e == cudaSuccess; first += batch) {
             const long long cnt = (n - first < batch) ? n - first : batch;
