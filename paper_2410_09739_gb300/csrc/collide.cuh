@@ -43,6 +43,13 @@ template <typename R>
 __device__ __forceinline__ R fmaR(R a, R b, R c) { return fma(a, b, c); }
 template <typename R>
 __device__ __forceinline__ R recipR(R a) { return R(1) / a; }
+// 1 / rho of a cell; NEWTON: a pair's takes the short form, as one cell's always does (pair.cuh).
+template <bool NEWTON = false, typename R>
+__device__ __forceinline__ R recip_rho(R rho)
+{
+    if constexpr (std::is_same<R, float>::value || (NEWTON && std::is_same<R, f2>::value)) return recip_newton(rho);
+    else return recipR(rho);
+}
 template <typename R>
 __device__ __forceinline__ R sqrtR(R a) { return sqrt(a); }
 template <typename R>
@@ -284,7 +291,7 @@ __device__ __forceinline__ bool collide_unit(R (&g)[27], const Rates<R>& rt, R F
     }
     const R drho = m000, rho = R(1) + drho;
     const bool ok = (rho > R(0)) && (rho < R(1e30));
-    const R inv = recipR(rho);
+    const R inv = recip_rho(rho);
     // minus the velocity (each of the transforms below subtracts)
     const R ninv = -inv;
     const R nx = (XF ? fmaR(R(0.5), Fx, m100) : m100) * ninv, ny = m010 * ninv, nz = m001 * ninv;
@@ -514,9 +521,7 @@ __device__ __forceinline__ bool collide_general(R (&g)[27], const Rates<R>& rt, 
     const R jy = ((S[6] - S[0]) + (S[7] - S[1])) + (S[8] - S[2]);
     const R jz = ((Dz[0] + Dz[1] + Dz[2]) + (Dz[3] + Dz[4] + Dz[5])) + (Dz[6] + Dz[7] + Dz[8]);
     const R rho = R(1) + drho;
-    R inv_rho;
-    if constexpr (NEWTON) inv_rho = recip_newton(rho);
-    else inv_rho = recipR(rho);
+    const R inv_rho = recip_rho<NEWTON>(rho);
     const bool ok = (rho > R(0)) && (rho < R(1e30));
     R ux, uy, uz;
     if (FORCE) {

@@ -72,7 +72,7 @@ __device__ __forceinline__ bool collide2(R (&g)[9], const Rates2<R>& rt, R Fx, R
     const R jx = S[2] - S[0];
     const R jy = (Dy[0] + Dy[1]) + Dy[2];
     const R rho = R(1) + drho;
-    const R inv_rho = recipR(rho);
+    const R inv_rho = recip_rho(rho);
     const bool ok = (rho > R(0)) && (rho < R(1e30));
     const R ux = (FORCE ? fmaR(R(0.5), Fx, jx) : jx) * inv_rho;
     const R uy = (FORCE ? fmaR(R(0.5), Fy, jy) : jy) * inv_rho;
