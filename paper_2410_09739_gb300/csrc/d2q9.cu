@@ -315,7 +315,7 @@ __device__ __forceinline__ void load2(const void* bufv, unsigned stride, int nx,
 // Product-form equilibrium deviation (equal to C(u)^-1 kappa^eq with the
 // Maxwellian central moments (1, 0, cs^2) per axis, times rho).  FP32 and 16-bit storage form
 //   g = [dr (A + a) + a] (B + b) + A b
-// on numbers that are sums of two fp32 values (field_math.cuh), rounded to fp32: the fp64 form was
+// on numbers that are sums of two fp32 values (field_math.cuh), rounded once to the stored type: the fp64 form was
 // bound by the fp64 pipe, 1.92 ms for 4096^2 cells in fp32 against 0.20 ms now; k_moments2d 1.67 ms against 0.53 ms.
 // FP64 storage, and cells out of those numbers' range, take the fp64 form.
 template <typename S>
@@ -356,8 +356,11 @@ __global__ void k_init2d(void* bufv, unsigned stride, unsigned n, const double* 
 #pragma unroll
                 for (int iy = 0; iy < 3; ++iy) {
                     const Dual<float> b = dual_mul(w6, Y.d[iy]);  // A b is this or four times it
-                    Store<S>::st(buf + (size_t)(ix + 3 * iy) * stride + c,
-                                 dual_sum(dual_mul(P, Y.f[iy]), ix == 1 ? dual_scale(b, 4.f) : b));
+                    const Dual<float> PY = dual_mul(P, Y.f[iy]), Ab = ix == 1 ? dual_scale(b, 4.f) : b;
+                    float g;
+                    if constexpr (sizeof(S) == 2) g = dual_sum_odd(PY, Ab);
+                    else g = dual_sum(PY, Ab);
+                    Store<S>::st(buf + (size_t)(ix + 3 * iy) * stride + c, g);
                 }
             }
             return;

@@ -116,6 +116,21 @@ __device__ __forceinline__ T dual_sum(Dual<T> a, Dual<T> b)
     return rn_add(s, rn_add(e, rn_add(a.l, b.l)));
 }
 
+// The sum rounded to fp32 by round-to-odd (the last bit set whenever anything is cut off), so that
+// rounding it once more, to a type of at most 22 significant bits, gives the sum rounded once
+// (S. Boldo and G. Melquiond, "Emulation of a FMA and correctly rounded sums: proved algorithms using
+// rounding to odd", IEEE Trans. Comput. 57 (2008)).
+__device__ __forceinline__ float dual_sum_odd(Dual<float> a, Dual<float> b)
+{
+    float s, e, h, l;
+    two_sum(a.h, b.h, s, e);
+    two_sum(s, rn_add(e, rn_add(a.l, b.l)), h, l);
+    const unsigned u = __float_as_uint(h);
+    // l points away from zero where it has h's sign: the odd neighbour is then the next larger magnitude
+    const unsigned odd = (__float_as_uint(l) ^ u) >> 31 ? u - 1u : u + 1u;
+    return l != 0.f && !(u & 1u) ? __uint_as_float(odd) : h;
+}
+
 // One axis of the product-form equilibrium at velocity u: the deviations d of the three factors
 // from the rest weights, (u^2 - u)/2, -u^2, (u^2 + u)/2, and the factors f = w1 + d.
 template <typename T>
