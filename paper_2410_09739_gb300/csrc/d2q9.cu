@@ -385,17 +385,22 @@ __global__ void k_moments2d(const void* buf, unsigned stride, int nx, int ny, in
             if (s % 3 != 1) x.add(s % 3 == 2 ? g[s] : -g[s]);
             if (s / 3 != 1) y.add(s / 3 == 2 ? g[s] : -g[s]);
         }
-        const double r = 1.0 + d.value(), inv = 1.0 / r;
-        // j / r from the reciprocal, with one correction by the quotient's remainder
-        auto over = [&](double j, double F) {
-            if (has_force) j += 0.5 * F;
-            const double q = j * inv;
-            return fma(fma(-q, r, j), inv, q);
-        };
-        if (rho) rho[c] = r;
-        if (ux) ux[c] = over(x.value(), Fx);
-        if (uy) uy[c] = over(y.value(), Fy);
-        return;
+        // sums that left fp32 (infinite, NaN or far beyond a density) and a density of zero go to the fp64
+        // form below, whose infinities and NaN they keep
+        const double r = 1.0 + d.value();
+        if (fabsf(d.s) + fabsf(x.s) + fabsf(y.s) < 1e30f && (__double2hiint(r) & 0x7ff00000) != 0) {
+            const double inv = 1.0 / r;
+            // j / r from the reciprocal, with one correction by the quotient's remainder
+            auto over = [&](double j, double F) {
+                if (has_force) j += 0.5 * F;
+                const double q = j * inv;
+                return fma(fma(-q, r, j), inv, q);
+            };
+            if (rho) rho[c] = r;
+            if (ux) ux[c] = over(x.value(), Fx);
+            if (uy) uy[c] = over(y.value(), Fy);
+            return;
+        }
     }
     double g[9];
     load2<S>(buf, stride, nx, ny, box, parity, c, g);

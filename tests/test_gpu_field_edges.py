@@ -1,5 +1,5 @@
 """Field kernels at the edges of their arithmetic: 16-bit storage in 2D rounded once from the exact
-equilibrium.
+equilibrium; infinite, huge and vanishing densities, which the sums of fp32 pairs leave to fp64.
 """
 import numpy as np
 import pytest
@@ -41,3 +41,55 @@ def test_init_2d_16_bit_rounds_once(prec, amp):
         want, tie = rounded((rho - 1) * ((A + p) * (B + q)) + (p * (B + q) + A * q), prec)
         assert np.array_equal(got[a][~tie], want[~tie]), a
         assert np.mean(tie) < 1e-6
+
+
+def same(a, b, rtol):
+    """Equal up to rtol, and infinite or NaN in the same places."""
+    with np.errstate(invalid="ignore"):
+        near = np.abs(a - b) <= rtol * np.abs(b)
+    return np.all((np.isnan(a) & np.isnan(b)) | (a == b) | near)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+@pytest.mark.parametrize("box", [False, True])
+@pytest.mark.parametrize("force", [False, True])
+def test_moments_2d_of_extreme_cells(prec, box, force):
+    """Infinite, NaN, huge and cancelling populations and a density of exactly zero: what fp64 sums and
+    divisions give; ordinary neighbours to the bound of test_moments_2d_are_fp64_sums."""
+    big = 2.0 ** 127
+    w = W2[:, 0, 0]
+    f = np.tile(W2, (1, 3, 4))
+    f[0, 0, 0] = np.inf
+    f[1, 0, 1] = -np.inf
+    f[5, 0, 2] = np.inf
+    f[6, 0, 2] = -np.inf
+    f[2, 0, 3] = np.nan
+    f[1, 1, 0] = f[2, 1, 0] = big            # the sum leaves fp32
+    f[1, 1, 1], f[3, 1, 1], f[5, 1, 1] = big, big, -big
+    f[0, 1, 2] = w[0] - 1.25                # density 0, momentum (0.25, 0)
+    f[1, 1, 2] = w[1] + 0.25
+    f[0, 1, 3] = w[0] - 1.0                 # density 0 at rest
+    f[3, 2, 0] += 0.125
+    f[:, 2, 1] *= 1.0 + 2.0 ** -6
+    F0 = (2.0 ** -8, -2.0 ** -9) if force else (0.0, 0.0)
+    with F.Lattice2D(4, 3, prec) as lat:
+        lat.set_params(0.7)
+        lat.set_force(*F0)
+        if box:
+            lat.set_boundary(F.FPCLBM_BC_BOX, 0.0)
+        lat.set_populations(f)
+        got = lat.moments()
+        g = lat.get_populations() - W2       # the stored deviations
+    with np.errstate(all="ignore"):
+        rho = 1.0 + g.sum(0)
+        # a product with a zero component is NaN for an infinite population, as in the fp64 kernel
+        j = [(e[:, None, None] * g).sum(0) + 0.5 * Fk for e, Fk in zip((EX2, EY2), F0)]
+        ref = [rho, j[0] / rho, j[1] / rho]
+    # densities of exactly zero: the stored deviations -1 - 0.25 + 0.25 have no rounding error
+    ref[0][1, 2:4] = 0.0
+    with np.errstate(all="ignore"):
+        ref[1][1, 2], ref[2][1, 2] = (0.25 + 0.5 * F0[0]) / np.float64(0.0), 0.5 * F0[1] / np.float64(0.0)
+        ref[1][1, 3], ref[2][1, 3] = (0.5 * np.array(F0)) / np.float64(0.0)
+    for x, y in zip(got, ref):
+        assert same(x[:2], y[:2], 1e-14), (x, y)
+        assert np.max(np.abs(x[2] - y[2])) <= 2e-15
