@@ -48,11 +48,7 @@ template <typename S>
 __device__ __forceinline__ void filter_fields(const FilterArgs& a, unsigned cell, double& r, double& u, double& v,
                                               double& w)
 {
-    if constexpr (std::is_same<S, double>::value) {
-        double g[27];
-        load_cell<S>(a.b, a.parity, cell, g);
-        fields_of(g, a.Fx, a.Fy, a.Fz, r, u, v, w);
-    } else {
+    if constexpr (!std::is_same<S, double>::value) {
         float g[27];
         load_cell<S>(a.b, a.parity, cell, g);
         float ds = 0.f, dc = 0.f, xs = 0.f, xc = 0.f, ys = 0.f, yc = 0.f, zs = 0.f, zc = 0.f;
@@ -64,20 +60,27 @@ __device__ __forceinline__ void filter_fields(const FilterArgs& a, unsigned cell
             if (ey != 0) sum2_add(ys, yc, ey > 0 ? g[s] : -g[s]);
             if (ez != 0) sum2_add(zs, zc, ez > 0 ? g[s] : -g[s]);
         }
-        r = 1.0 + (widen(ds) + widen(dc));
-        const double inv = 1.0 / r;
-        u = widen(xs) + widen(xc);
-        v = widen(ys) + widen(yc);
-        w = widen(zs) + widen(zc);
-        if (a.has_force) {
-            u += 0.5 * a.Fx;
-            v += 0.5 * a.Fy;
-            w += 0.5 * a.Fz;
+        // sums that left fp32 (infinite, NaN or far beyond a density) take the fp64 form
+        if (fabsf(ds) + fabsf(xs) + fabsf(ys) + fabsf(zs) < 1e30f) {
+            r = 1.0 + (widen(ds) + widen(dc));
+            const double inv = 1.0 / r;
+            u = widen(xs) + widen(xc);
+            v = widen(ys) + widen(yc);
+            w = widen(zs) + widen(zc);
+            if (a.has_force) {
+                u += 0.5 * a.Fx;
+                v += 0.5 * a.Fy;
+                w += 0.5 * a.Fz;
+            }
+            u *= inv;
+            v *= inv;
+            w *= inv;
+            return;
         }
-        u *= inv;
-        v *= inv;
-        w *= inv;
     }
+    double g[27];
+    load_cell<S>(a.b, a.parity, cell, g);
+    fields_of(g, a.Fx, a.Fy, a.Fz, r, u, v, w);
 }
 
 // Box filter.  A block takes `group` neighbouring coarse cells of a row, a thread one column of fine

@@ -4,6 +4,7 @@ equilibrium; infinite, huge and vanishing densities, which the sums of fp32 pair
 import numpy as np
 import pytest
 
+import oracle as O
 from paper_2410_09739_gb300 import fpclbm as F
 
 pytestmark = pytest.mark.gpu
@@ -93,3 +94,34 @@ def test_moments_2d_of_extreme_cells(prec, box, force):
     for x, y in zip(got, ref):
         assert same(x[:2], y[:2], 1e-14), (x, y)
         assert np.max(np.abs(x[2] - y[2])) <= 2e-15
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+@pytest.mark.parametrize("r", [2, 3])
+def test_sample_of_extreme_cells(prec, r):
+    """Coarse cells that hold one infinite population (density infinite, velocity NaN), two huge ones
+    whose sum leaves fp32, and a density of exactly zero moving along +x, as fp64 gives them; coarse
+    cells with no such cell next to them stay finite."""
+    n, big = 8 * r, 2.0 ** 127
+    f = O.init_equilibrium(np.ones((n, n, n)), *(0.02 * np.random.default_rng(5).uniform(-1, 1, (3, n, n, n))))
+    e = O.velocity_set()
+    w = W1[e[:, 0] + 1] * W1[e[:, 1] + 1] * W1[e[:, 2] + 1]
+    at = {tuple(int(c) for c in v): a for a, v in enumerate(e)}
+    rest, east = at[(0, 0, 0)], at[(1, 0, 0)]
+    f[rest, 0, 0, 0] = np.inf
+    f[rest, 0, 0, 3 * r] = f[east, 0, 0, 3 * r] = big
+    f[:, 0, 4 * r, 0] = w
+    f[rest, 0, 4 * r, 0] -= 1.25
+    f[east, 0, 4 * r, 0] += 0.25
+    with F.Lattice(n, n, n, prec) as lat:
+        lat.set_params(0.6)
+        lat.set_populations(f)
+        X, T = np.empty((512, 9), np.float32), np.empty(512, np.float32)
+        F.fpclbm_closure_sample(lat.h, r, 0.55, X, T)
+    X = X.reshape(8, 8, 8, 9)
+    assert np.all(np.isinf(X[0, 0, 0, :6])) and np.all(np.isnan(X[0, 0, 0, 6:]))
+    # density 2^128 + 1, momentum 2^127 along x: velocity 1/2 there, a mean of 1 / (2 r^3) and noise
+    assert np.all(np.isinf(X[0, 0, 3, :6]) | (np.abs(X[0, 0, 3, :6]) > 1e30))
+    assert abs(X[0, 0, 3, 6] - 0.5 / r ** 3) < 0.02 and np.all(np.abs(X[0, 0, 3, 7:]) < 0.02)
+    assert X[0, 4, 0, 6] == np.inf
+    assert np.all(np.isfinite(X[2:7]))
