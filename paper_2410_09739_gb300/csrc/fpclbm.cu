@@ -398,31 +398,46 @@ bool forced_launch(TuneChoice& c)
     return true;
 }
 
-// Whether the row-staged variant (stage.cuh) can run this handle: a single periodic box or
-// channel, fp32 arithmetic in the FP or MCM mode, 16- or 32-bit storage, rows of a multiple of
-// 16 bytes and at most 512 cells (tiles of 256 or 512 cells).
-bool stage_ok(const fpclbm* h)
+// Whether the row-staged variant (stage.cuh) covers this handle whatever its row length: a single
+// periodic box or channel, fp32 arithmetic in the FP or MCM mode, 16- or 32-bit storage.
+bool stage_family(const fpclbm* h)
 {
     if (h->ensemble || h->precision == FPCLBM_FP64) return false;
     const int kb = kernel_bc(h);
-    if (!(kb == BC_PERIODIC || kb == BC_WALLS_Y) || !plain_mode(mode_of(h))) return false;
-    const Box& b = h->boxes[0];
-    const size_t es = elem_size(h->precision);
-    return (b.nx * es) % 16 == 0 && b.nx <= 512;
+    return (kb == BC_PERIODIC || kb == BC_WALLS_Y) && plain_mode(mode_of(h));
+}
+
+// ... and can move its rows: a multiple of 16 bytes and at most 512 cells.
+bool stage_ok(const fpclbm* h)
+{
+    const int nx = h->boxes[0].nx;
+    return stage_family(h) && (nx * elem_size(h->precision)) % 16 == 0 && nx <= 512;
 }
 
 // Threads of a row-staged block: 4, 6 or 8 consumer warps and one producer warp.
-int stage_threads(const fpclbm* h)
+int stage_threads(const fpclbm* h) { return 32 * (stage_warps(h->boxes[0].nx) + 1); }
+
+// Whether a row-staged block with that many input stages fits this handle's rows and its device.
+bool stage_fits(const fpclbm* h, int stages)
 {
-    const int nx = h->boxes[0].nx;
-    return nx <= 256 ? 160 : nx <= 384 ? 224 : 288;
+    int optin = 0;
+    if (!stage_ok(h) || stages < 2 || stages > 6 ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device) != cudaSuccess)
+        return false;
+    return staged_block_bytes(stage_warps(h->boxes[0].nx), elem_size(h->precision), stages) <= (size_t)optin;
 }
 
+// What a choice holds for: besides the physics and the cell count the class of the rows, because rows of
+// odd length pair other cells on the odd step, and rows that cannot be staged, or only in wider tiles,
+// have other candidates.  Even rows whose variant is the usual one carry no suffix.
 std::string tune_key(const fpclbm* h)
 {
+    const int nx = h->boxes[0].nx;
+    const char* rows = h->ensemble ? "" : (nx & 1) ? "/odd" : !stage_family(h) ? "" : !stage_ok(h) ? "/plain"
+                       : stage_warps(nx) == 4 ? "" : stage_warps(nx) == 6 ? "/w384" : "/w512";
     char buf[160];
-    std::snprintf(buf, sizeof buf, "dev%d/p%d/bc%d/f%d/m%d/%s/%llu", h->device, h->precision, kernel_bc(h), force_kind(h),
-                  mode_of(h), h->ensemble ? "ens" : "box", (unsigned long long)(h->total_cells >> 20));
+    std::snprintf(buf, sizeof buf, "dev%d/p%d/bc%d/f%d/m%d/%s/%llu%s", h->device, h->precision, kernel_bc(h), force_kind(h),
+                  mode_of(h), h->ensemble ? "ens" : "box", (unsigned long long)(h->total_cells >> 20), rows);
     return buf;
 }
 
@@ -465,8 +480,8 @@ int autotune(fpclbm* h)
         if (pipe_ok)
             for (int minb : {2, 3, 4}) cands.push_back({128, minb, 0, 1});
         if (h->total_cells < pair_from) cands.push_back({128, 2, 0, 2});  // 4 blocks of 128 threads, 128 registers
-        if (stage_ok(h))  // row-staged paired variant with 2 or 3 input stages
-            for (int ns : {2, 3}) cands.push_back({stage_threads(h), 2, ns, 3});
+        for (int ns : {2, 3})  // row-staged paired variant with 2 or 3 input stages
+            if (stage_fits(h, ns)) cands.push_back({stage_threads(h), 2, ns, 3});
     } else if (learned_mode(mode_of(h)) && h->precision != FPCLBM_FP64 && fixed_walls) {
         // two cells per thread first (the collision on the packed fp32 pipe, the MLP once per
         // lane), then one cell per thread capped at 128 registers or uncapped
@@ -520,10 +535,9 @@ int autotune(fpclbm* h)
         std::lock_guard<std::mutex> lk(g_tune_mu);
         load_tune_file();
         auto it = g_tune_cache.find(tune_key(h));
-        // the key holds the cell count, not the row length: a row-staged choice of another box is no
-        // choice for one whose rows cannot be staged
-        if (it != g_tune_cache.end() && (it->second.pipe != 3 || stage_ok(h))) {
-            h->block = it->second.block;
+        // a row-staged choice from a file may be of other rows: one that does not fit these is no choice
+        if (it != g_tune_cache.end() && (it->second.pipe != 3 || stage_fits(h, it->second.grid))) {
+            h->block = it->second.pipe == 3 ? stage_threads(h) : it->second.block;
             h->minb = it->second.minb;
             h->grid = it->second.grid;
             h->pipe = it->second.pipe;

@@ -44,6 +44,15 @@ cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, 
     return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
+// Row-staged variant (stage.cuh): consumer warps of a block, each 64 cells of its tile, for rows of nx
+// cells, and the shared memory of a block with nsi input stages.
+constexpr unsigned kStageOut = 2;  // output stages (a power of two: stage and phase by shifts)
+__host__ __device__ constexpr int stage_warps(int nx) { return nx <= 256 ? 4 : nx <= 384 ? 6 : 8; }
+__host__ __device__ constexpr size_t staged_block_bytes(int warps, size_t elem, int nsi)
+{
+    return (size_t)(nsi + kStageOut) * (27 * 64 * warps * elem + 16) + 16;
+}
+
 // One time step of a single box.  odd selects the AA-pattern parity (0: own
 // slots, 1: neighbour slots), bc the boundary kind (BC_*), force the FORCE_* kind
 // of the body force, mode one of the MODE_* collision modes (common.cuh).

@@ -49,7 +49,6 @@ namespace fpc {
 
 inline StepArgs<f2> pair_args(const StepArgs<float>& a);  // step_kernel.cuh
 constexpr int kStageFlagTimeout = 2;
-constexpr unsigned kStageOut = 2;  // output stages (a power of two: stage and phase by shifts)
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -515,10 +514,9 @@ template <typename S, bool ODD, int BC, int FORCE, int MODE, int NCW>
 cudaError_t step_go_stage_ncw(const StepArgs<float>& a, int nsi, cudaStream_t st)
 {
     constexpr int TC = 64 * NCW;
-    constexpr int nso = kStageOut;
     const int R = stage_rows(a.nx, a.ny, TC);
     const int threads = 32 * (NCW + 1);
-    const size_t smem = (size_t)(nsi + nso) * 27 * TC * sizeof(S) + 16 * (size_t)(nsi + nso) + 16;
+    const size_t smem = staged_block_bytes(NCW, sizeof(S), nsi);
     auto kern = k_step_stage<S, ODD, BC, FORCE, MODE, NCW>;
     // resident blocks per SM for the last shared-memory size this instantiation launched with,
     // on the device of that launch (a benign race: every thread computes the same values)
@@ -559,9 +557,11 @@ template <typename S, bool ODD, int BC, int FORCE, int MODE>
 cudaError_t step_go_stage(const StepArgs<float>& a, int nsi, cudaStream_t st)
 {
     if ((a.nx * sizeof(S)) % 16 != 0 || a.nx > 512 || a.nx < 2 || nsi < 2 || nsi > 6) return cudaErrorInvalidValue;
-    if (a.nx <= 256) return step_go_stage_ncw<S, ODD, BC, FORCE, MODE, 4>(a, nsi, st);
-    if (a.nx <= 384) return step_go_stage_ncw<S, ODD, BC, FORCE, MODE, 6>(a, nsi, st);
-    return step_go_stage_ncw<S, ODD, BC, FORCE, MODE, 8>(a, nsi, st);
+    switch (stage_warps(a.nx)) {
+        case 4: return step_go_stage_ncw<S, ODD, BC, FORCE, MODE, 4>(a, nsi, st);
+        case 6: return step_go_stage_ncw<S, ODD, BC, FORCE, MODE, 6>(a, nsi, st);
+        default: return step_go_stage_ncw<S, ODD, BC, FORCE, MODE, 8>(a, nsi, st);
+    }
 }
 
 }  // namespace fpc
