@@ -211,28 +211,42 @@ inline StepArgs<f2> pair_args(const StepArgs<float>& a)
     return p;
 }
 
+// L2 of the GB300 (129 MB); populations beyond it come from HBM every step.
+constexpr unsigned long long kL2Bytes = 129000000;
+
+// Resident blocks per SM the registers are capped for: four (128 registers hold two cells without
+// spilling; the learned modes spill about 90 bytes, 2.5 % faster than three blocks at 168), or five for
+// - the even step without force or moving wall (vector accesses, no neighbour table, no source terms), which
+//   fits 96 registers without spilling;
+// - 16-bit storage with a force along x, where five blocks spill and pay all the same in larger boxes
+//   (periodic boxes, channels and half channels, step pairs against four blocks):
+//   even step (28 bytes), from 2^18 cells: 64^3 -1.8 to +0.6 %, 192x96x96 -1.2 to -2.6 %, 384x192x192 -1.9 to
+//   -6.3 % (48^3 up to 3.5 % slower);
+//   odd step of neighbouring cells (148 bytes), FP and MCM modes, populations beyond L2: walls 384x192x192
+//   -0.6 to -3.2 %, periodic FP -1.0 to -1.5 %; not periodic MCM (+0.0 to +0.7 %), boxes that stay in L2
+//   (192x96x96 up to 7.3 % slower) or odd rows (cells c, c + N/2: up to 16 % slower).
+// fp32 with a force along x is bound by HBM: five blocks on its even step gave FP and MCM +0.4 to -0.5 %
+// and the Smagorinsky mode +0.5 to +1.2 %.
 template <typename S, bool ODD, int BC, int FORCE, int MODE, int MINB>
 cudaError_t step_go_pair(const StepArgs<float>& a, cudaStream_t st)
 {
     const unsigned half = (a.ncells + 1) / 2;
-    // the even step without force or moving wall (vector accesses, no neighbour table, no source
-    // terms) fits in 96 registers without spilling: one block more per SM.  With a force along x it
-    // spills 28 bytes there and is faster all the same (384x192x192 bf16 channel: 326 -> 281 us;
-    // fp32, bound by HBM: unchanged); 16-bit storage gains from the fifth block on the odd step too
-    // (148 bytes of spills; same channel 402 -> 384 us; not the fp32 LES, 177 -> 179).  The learned
-    // modes run four blocks (128 registers, about 90 bytes of spills: 2.5 % faster than three blocks
-    // at 168)
-    constexpr bool LID = BC == BC_WALLS_Y_LID || BC == BC_BOX_LID;
-    constexpr bool WIDE_ODD = FORCE == FORCE_X && sizeof(S) == 2 && plain_mode(MODE);
-    constexpr bool NARROW = (ODD && !WIDE_ODD) || FORCE == FORCE_ANY || LID;
-    constexpr int BLOCKS = learned_mode(MODE) ? 4 : NARROW ? 2 * MINB : 2 * MINB + 1;
     const unsigned grid = (half + 127) / 128;
+    constexpr bool LID = BC == BC_WALLS_Y_LID || BC == BC_BOX_LID;
+    constexpr bool X16 = FORCE == FORCE_X && sizeof(S) == 2 && !LID && !learned_mode(MODE);
+    constexpr int CAP = learned_mode(MODE) ? 4 : !ODD && FORCE == FORCE_NONE && !LID ? 2 * MINB + 1 : 2 * MINB;
     // neighbouring cells on the odd step: nx even (rows hold whole pairs); the closed box only with
     // fp32 storage (its per-cell x-wall tests spill with 16-bit unpacking)
     constexpr bool ADJ_OK = ODD && (BC != BC_BOX_LID || sizeof(S) == 4);
-    if (ADJ_OK && (a.nx & 1) == 0)
-        return launch_chained(k_step_pair<S, ODD, BC, FORCE, MODE, BLOCKS, ADJ_OK>, grid, 128, 0, st, pair_args(a), half);
-    return launch_chained(k_step_pair<S, ODD, BC, FORCE, MODE, BLOCKS, false>, grid, 128, 0, st, pair_args(a), half);
+    const bool adj = ADJ_OK && (a.nx & 1) == 0;
+    if constexpr (X16 && (!ODD || (plain_mode(MODE) && !(BC == BC_PERIODIC && eq_mode(MODE))))) {
+        const bool five = ODD ? adj && 27ull * sizeof(S) * a.ncells > kL2Bytes : a.ncells >= (1u << 18);
+        if (five)
+            return launch_chained(k_step_pair<S, ODD, BC, FORCE, MODE, 2 * MINB + 1, ADJ_OK>, grid, 128, 0, st,
+                                  pair_args(a), half);
+    }
+    if (adj) return launch_chained(k_step_pair<S, ODD, BC, FORCE, MODE, CAP, ADJ_OK>, grid, 128, 0, st, pair_args(a), half);
+    return launch_chained(k_step_pair<S, ODD, BC, FORCE, MODE, CAP, false>, grid, 128, 0, st, pair_args(a), half);
 }
 
 template <typename S, typename R, bool ODD, int BC, int FORCE, int MODE, int MINB>
