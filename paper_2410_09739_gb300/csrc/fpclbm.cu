@@ -455,6 +455,15 @@ int autotune(fpclbm* h)
     // paired variant (two cells per thread, packed fp32): fp32 arithmetic, every boundary kind
     const bool pair_ok = fp32_math;
     const bool pair_smag = h->precision != FPCLBM_FP64 && md == MODE_SMAG_R1;
+    // The first candidate runs boxes too small to tune: two cells per thread where the step is longer than
+    // its latency (fp32, us a step, one / two cells: 32^3 2.20 / 2.25, 48^3 4.56 / 3.59, 64^3 8.09 / 6.55,
+    // 96^3 29.8 / 23.8); rows of odd length pair cells c, c + N/2 and gain later (45x37x53 3.93 / 4.12,
+    // 63x65x67 8.6 / 7.9), and so does the closed box, whose odd step tests six walls.  Two cells over one,
+    // all storage types, rates and forces: 40x41x40 0.85 to 1.00 (closed box 1.00 to 1.08), 44x46x45 0.82 to
+    // 1.00 (1.02 to 1.12), 48^3 0.73 to 0.88 (0.92 to 0.98), odd rows 41x40x40 0.96 to 1.23, 63x65x65 0.82 to
+    // 0.96; Smagorinsky mode 8^3 1.3 to 1.5, 32^3 1.10 to 1.17, 40x41x40 0.93 to 1.04, 48^3 0.78 to 0.82, odd
+    // rows 41x40x40 1.06 to 1.17, 63x65x65 0.89 to 0.94.
+    const unsigned long long pair_from = (h->boxes[0].nx & 1) ? 1ull << 18 : kb == BC_BOX_LID ? 3ull << 15 : 1ull << 16;
     if (h->ensemble) {
         for (int minb : {2, 3})
             for (int block : {128, 256}) {
@@ -469,11 +478,6 @@ int autotune(fpclbm* h)
             cands.push_back({128, minb, (int)h->ntiles, 2});
         }
     } else if (fp32_math) {
-        // the first candidate runs boxes too small to tune: two cells per thread where the step is
-        // longer than its latency (fp32, us a step, one / two cells: 32^3 2.20 / 2.25, 48^3 4.56 /
-        // 3.59, 64^3 8.09 / 6.55, 96^3 29.8 / 23.8); rows of odd length pair cells c, c + N/2 and
-        // gain later (45x37x53 3.93 / 4.12, 63x65x67 8.6 / 7.9)
-        const unsigned long long pair_from = (h->boxes[0].nx & 1) ? 1ull << 18 : 1ull << 16;
         if (h->total_cells >= pair_from) cands.push_back({128, 2, 0, 2});
         for (int minb : {2, 3, 4})
             for (int block : {128, 256}) cands.push_back({block, minb, 0, 0});
@@ -489,7 +493,7 @@ int autotune(fpclbm* h)
         for (int minb : {2, 1})
             for (int block : {128, 256}) cands.push_back({block, minb, 0, 0});
     } else {
-        if (pair_smag) cands.push_back({128, 2, 0, 2});
+        if (pair_smag && h->total_cells >= pair_from) cands.push_back({128, 2, 0, 2});
         // fp64 first with blocks of one warp: the step is bound by the fp64 pipe of the SM with most
         // cells, and small blocks share a small box out evenly (32^3, us a step with blocks of 128,
         // 64, 32: 26.7, 26.6, 23.9; 16^3 14.2, 12.5, 12.6; equal from 45x37x53 on)
