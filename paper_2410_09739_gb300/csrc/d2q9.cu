@@ -468,15 +468,17 @@ inline Args2<f2> pair_args(const Args2<float>& a)
     return p;
 }
 
-// Boxes below this many cells run one cell per thread: their step is latency, not throughput
-// (256^2 fp32 2.0 us a step with one cell per thread, 64^2 1.7).
-constexpr unsigned kPair2Cells = 1u << 16;
+// Boxes below this many cells run one cell per thread: their step is latency, not throughput.  Two cells
+// over one, periodic and closed boxes, both modes, with and without force, fp32 / 16-bit storage: 256^2 1.05 to
+// 1.13 / 1.00 to 1.03, 364^2 0.91 to 1.01 / 0.89 to 0.97, 400^2 0.90 to 0.98, 512^2 0.84 to 0.98; rows of odd
+// length, whose odd step stays with one cell: 363^2 1.00 to 1.09, 511x513 0.92 to 0.98.
+__host__ constexpr unsigned pair2_from(unsigned nx) { return nx & 1 ? 1u << 18 : 1u << 17; }
 
 template <typename S, typename R, bool BOX, bool ODD, bool FORCE, int MODE>
 cudaError_t step2d_one(const Args2<R>& a, cudaStream_t st)
 {
     if constexpr (sizeof(R) == 4) {  // fp32 arithmetic
-        if (a.ncells >= kPair2Cells && !(ODD && (a.nx & 1)))
+        if (a.ncells >= pair2_from(a.nx) && !(ODD && (a.nx & 1)))
             return launch_chained(k_step2d_pair<S, ODD, FORCE, MODE, BOX>, ((a.ncells + 1) / 2 + 127) / 128, 128, 0, st,
                                   pair_args(a));
     }
