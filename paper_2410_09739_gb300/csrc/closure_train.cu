@@ -83,28 +83,29 @@ __device__ __forceinline__ void filter_fields(const FilterArgs& a, unsigned cell
     fields_of(g, a.Fx, a.Fy, a.Fz, r, u, v, w);
 }
 
-// Box filter.  A block takes `group` neighbouring coarse cells of a row, a thread one column of fine
-// cells along y and z, so a warp reads consecutive fine cells of each slot row; the columns of a
+// Box filter.  A block takes `group` consecutive coarse cells, over the ends of rows, a thread one column of
+// fine cells along y and z, so a warp reads consecutive fine cells of each slot row; the columns of a
 // coarse cell are then summed through shared memory.  (One thread per coarse cell, all in fp64, read
-// every r-th cell and kept the fp64 pipe busy with about 180 operations per fine cell: 5.48 ms for 256^3 fp32 cells, r = 4, against 0.91 ms.)
+// every r-th cell and kept the fp64 pipe busy with about 180 operations per fine cell: 5.48 ms for 256^3
+// fp32 cells, r = 4, against 0.91 ms.  Blocks that ended with the row left most threads idle in short rows; whole
+// calls, fp32 / fp64 storage: 8x256x256, r = 2, 0.45 -> 0.17 / 1.30 -> 0.32 ms; 4x512x512, r = 4, 1.05 -> 0.09 /
+// 4.33 -> 0.36; 96^3, r = 4, 0.12 -> 0.08 / 0.28.)
 constexpr int kFilterThreads = 256;
 
 template <typename S>
 __global__ void __launch_bounds__(kFilterThreads) k_cl_filter(FilterArgs a)
 {
-    __shared__ double sh[10][kFilterThreads];
-    const unsigned groups = ((unsigned)a.cx + a.group - 1) / a.group;  // per coarse row
-    const unsigned row = blockIdx.x / groups, X0 = (blockIdx.x - row * groups) * a.group;
-    const unsigned Y = row % a.cy, Z = row / a.cy;
-    const unsigned cells = min((unsigned)a.group, (unsigned)a.cx - X0);  // coarse cells of this block
-    const unsigned cols = cells * a.r, tid = threadIdx.x;
+    extern __shared__ double cl_sums[];  // [10][threads]
+    const unsigned nc = (unsigned)a.cx * a.cy * a.cz, r = (unsigned)a.r, tid = threadIdx.x, nt = blockDim.x;
+    const unsigned first = blockIdx.x * a.group, cells = min((unsigned)a.group, nc - first);
     double s[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (unsigned c = tid; c < cols; c += blockDim.x)  // more than one column only if group == 1
-        for (int k = 0; k < a.r; ++k)
-            for (int j = 0; j < a.r; ++j) {
-                const unsigned x = X0 * a.r + c, y = Y * a.r + j, z = Z * a.r + k;
+    for (unsigned c = tid; c < cells * r; c += nt) {  // more than one column only if group == 1
+        const unsigned lc = c / r, row = (first + lc) / a.cx, Z = row / a.cy;
+        const unsigned x = (first + lc - row * a.cx) * r + (c - lc * r), y0 = (row - Z * a.cy) * r, z0 = Z * r;
+        for (unsigned k = 0; k < r; ++k)
+            for (unsigned j = 0; j < r; ++j) {
                 double rho, u, v, w;
-                filter_fields<S>(a, x + (unsigned)a.b.nx * (y + (unsigned)a.b.ny * z), rho, u, v, w);
+                filter_fields<S>(a, x + (unsigned)a.b.nx * (y0 + j + (unsigned)a.b.ny * (z0 + k)), rho, u, v, w);
                 s[0] += rho;
                 s[1] += u;
                 s[2] += v;
@@ -116,15 +117,17 @@ __global__ void __launch_bounds__(kFilterThreads) k_cl_filter(FilterArgs a)
                 s[8] += u * w;
                 s[9] += v * w;
             }
-    for (int q = 0; q < 10; ++q) sh[q][tid] = s[q];
+    }
+    for (int q = 0; q < 10; ++q) cl_sums[q * nt + tid] = s[q];
     __syncthreads();
-    const unsigned nc = (unsigned)a.cx * a.cy * a.cz, per = min((unsigned)a.r, (unsigned)blockDim.x);
+    const unsigned per = min(r, nt);
     const double inv = 1.0 / ((double)a.r * a.r * a.r);
-    for (unsigned i = tid; i < 10 * cells; i += blockDim.x) {
+    for (unsigned i = tid; i < 10 * cells; i += nt) {
         const unsigned q = i / cells, c = i - q * cells;
-        double t = 0;
-        for (unsigned m = 0; m < per; ++m) t += sh[q][c * per + m];
-        a.acc[(size_t)q * nc + (X0 + c) + (unsigned)a.cx * row] = t * inv;
+        const double* p = cl_sums + q * nt + c * per;
+        double t = p[0];
+        for (unsigned m = 1; m < per; ++m) t += p[m];
+        a.acc[(size_t)q * nc + first + c] = t * inv;
     }
 }
 
@@ -839,16 +842,24 @@ extern "C" int fpclbm_closure_sample(fpclbm_t h, int r, double tau_coarse, float
     g.walls = walls;
     g.div_nx = make_fastdiv((unsigned)B.nx);
     g.div_nxny = make_fastdiv((unsigned)(B.nx * B.ny));
-    const int group = std::max(1, std::min(cx, kFilterThreads / r));
+    // threads of a filter block: few enough that every SM has two, but a column each where one cell has
+    // more than a warp's
+    int threads = kFilterThreads, group = std::max(1, threads / r);
+    while (threads > 32 && threads / 2 >= r && (nc + group - 1) / group < 2 * (size_t)h->sm_count) {
+        threads /= 2;
+        group = threads / r;
+    }
+    threads = std::min(kFilterThreads, (group * r + 31) / 32 * 32);
+    const size_t smem = 10 * sizeof(double) * threads;
     const int force = h->F[0] != 0.0 || h->F[1] != 0.0 || h->F[2] != 0.0;
     FilterArgs fa{g, (int)(h->steps & 1), r, cx, cy, cz, group, force, h->F[0], h->F[1], h->F[2], acc};
     const unsigned blocks = (unsigned)((nc + 127) / 128);
-    const unsigned fblocks = (unsigned)((cx + group - 1) / group) * (unsigned)cy * (unsigned)cz;
+    const unsigned fblocks = (unsigned)((nc + group - 1) / group);
     switch (h->precision) {
-        case FPCLBM_FP64: k_cl_filter<double><<<fblocks, kFilterThreads, 0, h->stream>>>(fa); break;
-        case FPCLBM_FP32: k_cl_filter<float><<<fblocks, kFilterThreads, 0, h->stream>>>(fa); break;
-        case FPCLBM_FP32_STORE_FP16: k_cl_filter<__half><<<fblocks, kFilterThreads, 0, h->stream>>>(fa); break;
-        default: k_cl_filter<__nv_bfloat16><<<fblocks, kFilterThreads, 0, h->stream>>>(fa); break;
+        case FPCLBM_FP64: k_cl_filter<double><<<fblocks, threads, smem, h->stream>>>(fa); break;
+        case FPCLBM_FP32: k_cl_filter<float><<<fblocks, threads, smem, h->stream>>>(fa); break;
+        case FPCLBM_FP32_STORE_FP16: k_cl_filter<__half><<<fblocks, threads, smem, h->stream>>>(fa); break;
+        default: k_cl_filter<__nv_bfloat16><<<fblocks, threads, smem, h->stream>>>(fa); break;
     }
     k_cl_label<<<blocks, 128, 0, h->stream>>>(acc, cx, cy, cz, walls, tau_coarse, dX, dT);
     e = cudaGetLastError();

@@ -19,7 +19,9 @@ pytestmark = pytest.mark.gpu
 FORCE = (1e-5, -2e-5, 1e-5)
 
 
-@pytest.mark.parametrize("r,coarse", [(2, (129, 2, 2)), (3, (7, 2, 2)), (4, (66, 2, 2)), (5, (53, 3, 2)), (40, (3, 2, 2))])
+@pytest.mark.parametrize("r,coarse", [(2, (129, 2, 2)), (3, (7, 2, 2)), (4, (66, 2, 2)), (5, (53, 3, 2)), (40, (3, 2, 2)),
+                                      # short rows, blocks of one warp and of eight
+                                      (1, (2, 5, 4)), (2, (2, 40, 40)), (3, (5, 9, 50)), (2, (8, 72, 72)), (1, (3, 210, 130))])
 @pytest.mark.parametrize("prec", ["fp64", "fp32", "fp16", "bf16"])
 @pytest.mark.parametrize("walls", [0, 1])
 def test_every_column(r, coarse, prec, walls):
