@@ -487,9 +487,15 @@ int autotune(fpclbm* h)
         for (int ns : {2, 3})  // row-staged paired variant with 2 or 3 input stages
             if (stage_fits(h, ns)) cands.push_back({stage_threads(h), 2, ns, 3});
     } else if (learned_mode(mode_of(h)) && h->precision != FPCLBM_FP64 && fixed_walls) {
-        // two cells per thread first (the collision on the packed fp32 pipe, the MLP once per
-        // lane), then one cell per thread capped at 128 registers or uncapped
-        cands.push_back({128, 2, 0, 2});
+        // two cells per thread first (the collision on the packed fp32 pipe, the MLP once per lane),
+        // then one cell per thread capped at 128 registers or uncapped.  A pair evaluates the MLP twice in
+        // a row, so boxes too small to tune run one cell: uncapped while one wave of its blocks (two per SM)
+        // holds the box, then capped, in 16-bit storage up to 2^19 cells.  Us a step, uncapped / capped / pair,
+        // periodic and channels, unit and general rates, without and with force: 17x15x16 3.5-4.1 / 3.9-4.9 /
+        // 6.3-10.2, 33x31x32 4.3-4.8 / 4.5-5.4 / 6.5-10.6, 40x41x40 7.4-8.3 / 6.1-7.2 / 7.7-11.7, 64^3 capped 17.3-20.8
+        // (16-bit 17.6-21.0), pair 18.3-22.7 (18.0-20.9); 100^3 62-74 (60-72), pair 62-76 (57-67).
+        if (h->total_cells <= 256ull * h->sm_count) cands.push_back({128, 1, 0, 0});
+        else if (h->total_cells >= (h->precision == FPCLBM_FP32 ? 1ull << 20 : 1ull << 19)) cands.push_back({128, 2, 0, 2});
         for (int minb : {2, 1})
             for (int block : {128, 256}) cands.push_back({block, minb, 0, 0});
     } else {
