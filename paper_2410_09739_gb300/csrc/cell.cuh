@@ -362,7 +362,8 @@ __device__ __forceinline__ void move_inner(S* __restrict__ buf, const CellGeom& 
 // of the first cell, x = 0 for one at x - 1); a bounce-back redirect stays
 // within the cells' own slots (plus 1).  In the closed box the x walls give
 // the two cells different tests for e_x != 0, so there the second cell's
-// address is formed from its own test.  Not for the half channel.
+// address is formed from its own test.  In the half channel a link through
+// the symmetry plane moves in x like any other; one into the wall does not.
 template <typename S, int BC, int FORCE, int MODE>
 __device__ __forceinline__ void update_pair_odd_adj(S* __restrict__ buf, const CellGeom& G, unsigned t,
                                                     const Rates<f2>& rt, f2 Fx, f2 Fy, f2 Fz,

@@ -25,7 +25,7 @@ __device__ __forceinline__ R both(float v)
 }
 
 // One shear rate for all five of a box (the same values as Rates::keep and Rates::unit of a single
-// box with that rate, so both advance a box bit for bit alike).
+// box with that rate, so both advance a box bit for bit alike when both run one cell per thread or both two).
 template <int FORCE, int MODE, typename R>
 __device__ __forceinline__ Shear<R> box_shear(const EnsBox& B)
 {
